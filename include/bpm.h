@@ -147,22 +147,20 @@ int bpm_set_strain(bpm_plan_t plan, int32_t kind, const double* ux_um,
  *   BPM_SPLIT_FOREST_RUTH: a = (0, t, 1-2t, t), b = (t/2, (1-t)/2, (1-t)/2,
  *                          t/2), t = 1/(2 - 2^(1/3)).
  * FP64 plans take every method.  FP32 (fused) plans take the first-order
- * step, and for nx <= 4096 Verlet (half-step couplings on either side of
- * the full-step propagation; at nx = 4096 one 4-CTA half-band split per
- * solve while every solve gets four SMs, else one 2-CTA cluster per solve
- * while every solve gets two SMs and 512 <= nx != 2048, else one CTA per
- * solve) and Forest-Ruth (the leading coupling, then three
+ * step, Verlet (half-step couplings on either side of the full-step
+ * propagation) and Forest-Ruth (the leading coupling, then three
  * propagate-and-couple stages with the propagator increments of t dz and
- * (1 - 2t) dz, tabulated here once; at nx = 4096 one 4-CTA half-band split
- * per solve while every solve gets four SMs, for 512 <= nx <= 4096 one
- * 2-CTA cluster per solve while every solve gets two SMs, else one CTA per
- * solve), for
- * nx = 8192 Verlet and Forest-Ruth on one split-band cluster per solve, and
- * for nx = 16384 Verlet (one split-band cluster per solve) and Forest-Ruth
- * stage by stage (per step a coupling launch and three one-step launches
- * of the first-order split-band kernel with the stage's tables; several
- * times slower, and refused under stream capture; BPM_FUSED_LAYOUT=staged
- * takes it at nx = 8192 too); 3D plans take the first-order step
+ * (1 - 2t) dz, tabulated here once).  Rows of nx >= 512 march in one launch,
+ * each spread over a cluster of 4 to 16 SMs while all rows of the plan run
+ * at once that way (see bpm_launch_shape); more rows take one 4-CTA or 2-CTA
+ * cluster per row while every row gets those SMs, else one CTA per row (nx
+ * <= 4096) or one split-band cluster per row (nx >= 8192, Forest-Ruth for
+ * nx = 8192 only).  BPM_FUSED_LAYOUT=staged (or any other value at nx =
+ * 16384) marches Forest-Ruth stage by stage there: per step a coupling
+ * launch and three one-step launches, ten times slower.  Forest-Ruth plans
+ * of nx = 16384 are refused under stream capture in either form (and
+ * nx = 8192 plans while BPM_FUSED_LAYOUT=staged
+ * is set); 3D plans take the first-order step
  * and Verlet (the row kernel, which holds both bands of a line, applies the
  * half-step couplings); other combinations return BPM_ERR_INVALID.
  * bpm_submit takes FP32 plans set to Verlet or Forest-Ruth: their rows
@@ -350,25 +348,28 @@ int bpm_march_f64_noalloc(void* d_psi, int32_t nx, int32_t n_rows, const void* d
                           int32_t n_end, void* stream);
 
 /* Launch shape of the plan's last FP32 march (the fused kernels of the
- * step of Eq. fov10): *layout = 10 the Forest-Ruth step on one 2-CTA
- * cluster per row (512 <= nx <= 4096, while every row gets two SMs), 9 the
- * Forest-Ruth step on one 4-CTA
- * cluster per row (nx = 4096 half-band split, while every row gets four
- * SMs; nx = 8192 split band), 8 the nx = 4096 half-band split with 16
+ * step of Eq. fov10).  Rows of nx >= 512 are spread over clusters of 4, 8 or
+ * 16 CTAs while that is the faster form (nx = 512 to about 250 rows, 1024
+ * to 136, 2048 to 72, 4096 to 36, 8192 to 28, 16384 always but for 15 rows);
+ * they report the code of their size's cluster form below.  *layout = 10
+ * the Forest-Ruth step on one cluster per row (512 <= nx <= 4096), 9 the
+ * Forest-Ruth step on one cluster per row (nx = 4096 and 8192: 4-CTA
+ * half-band split, split band), 8 the nx = 4096 half-band split with 16
  * points per thread (forced by BPM_FUSED_LAYOUT=split16), 7 the Forest-Ruth
- * step stage by stage (nx = 16384, or nx = 8192 with
- * BPM_FUSED_LAYOUT=staged), 6 one CTA per row with the Forest-Ruth step (plans set to
- * BPM_SPLIT_FOREST_RUTH), 5 one split-band cluster per row with
- * the Verlet step (nx = 4096, 8192, 16384), 4 one 2-CTA cluster per row with the Verlet
- * step, 3 one CTA per row with the Verlet step (plans set to
- * BPM_SPLIT_VERLET), 2 one 4-CTA cluster per row (nx = 4096 as
- * two half-band parts per band; the rule while every row gets four SMs),
- * 1 one 2-CTA cluster per row, 0 one CTA per row, -1 chosen by the fixed
- * rule (2-CTA cluster while every row gets two SMs, else one CTA per row);
+ * step of nx = 16384 (or of nx = 8192 stage by stage with
+ * BPM_FUSED_LAYOUT=staged), 6 one CTA per row with the Forest-Ruth step, 5
+ * one cluster per row with the Verlet step (nx = 4096, 8192, 16384), 4 one
+ * cluster per row with the Verlet step (nx = 512, 1024; 2-CTA clusters at
+ * every nx <= 4096), 3 the Verlet step of nx = 2048 and on one CTA per row,
+ * 2 one cluster per row (nx = 4096: spread, or two half-band parts per band
+ * on four CTAs; smaller nx: spread batches), 1 one 2-CTA cluster per row,
+ * 0 one CTA per row, -1 chosen by the fixed rule (spread, 2-CTA cluster while
+ * every row gets two SMs, else one CTA per row).  BPM_FUSED_LAYOUT, set to any
+ * value, keeps rows off the spread form.
  * *chunk = steps per launch of the rotation schedule (more rows than one
- * launch keeps resident), 0 for a single launch.  A batch march with a
- * choice of shapes (the layouts above for up to one row per two SMs at
- * 512 <= nx <= 4096, or rotation chunks of 64..512 steps) times each on a
+ * launch keeps resident), 0 for a single launch.  A batch march that is not
+ * spread and has a choice of shapes (the layouts above for up to one row per
+ * two SMs at 512 <= nx <= 4096, or rotation chunks of 64..512 steps) times each on a
  * short march of a scratch copy of the state the first time a given
  * (nx, rows) is marched, blocking the host for those trials, and keeps the
  * fastest for the process; BPM_AUTOTUNE=0 in the environment or a single

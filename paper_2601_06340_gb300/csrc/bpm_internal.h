@@ -64,6 +64,8 @@ static_assert(sizeof(SepRow) == 96, "bulk-copied rows: a multiple of 16 bytes");
 struct RowDescF32 {
   float2* state;            // [2][N] raw envelopes (common phase removed)
   const float2* prop;       // [2][N] (P(q)-1)/N in the FFT's output order
+  const float2* prop_nat;   // spread rows: [tables][2][N] (P(q)-1)/N in natural frequency
+                            // order, else null
   const float2* prop_split; // N = 4096 rows on a 4-CTA cluster: [2][3][N/2] circulant
                             // tables of the half-band split, else null
   const float2* phasor;     // [nz][N] exp(i h u_x), (0,0) outside the crystal; null in
@@ -146,6 +148,8 @@ struct bpm_plan_s {
   bool sep_slices = false;        // the last prepared slices are separable
   void* d_prop = nullptr;         // [B][2][nx] c64 (delta form) or c128
   void* d_prop_split = nullptr;   // [B][2][3][nx/2] c64: N = 4096 half-band split tables
+  void* d_prop_nat = nullptr;     // [B][2][nx] c64: (P - 1)/N in natural frequency order
+                                  // (spread kernels)
   void* d_tw = nullptr;           // FP32: float4 [nx] hi/lo; FP64: double2 [nx]
   void* d_state = nullptr;        // [B][2][nx] c64 / c128
   void* d_state2 = nullptr;       // FP64 ping-pong buffer
@@ -167,6 +171,8 @@ struct bpm_plan_s {
   void* d_stage_prop_split = nullptr;   // FP32 Forest-Ruth on the split kernels (nx = 4096
                                         // half-band split, nx = 8192 split band): float2
                                         // [B][2 tables][split table in thread order]
+  void* d_stage_prop_nat = nullptr;     // FP32 Forest-Ruth on the spread kernels: float2
+                                        // [B][2 tables][2][nx] in natural frequency order
   size_t device_bytes = 0;
   int pending = 0;                // tickets not yet finished
   // launch shape of the last fused march: layout 1 cluster / 0 CTA / -1 rule,
@@ -187,11 +193,16 @@ int cuda_fail(cudaError_t e, const char* what);
 // Plan math (plan.cpp).
 int validate_problem(const bpm_problem* p, std::string* why);
 void compute_energy_consts(bpm_plan_s* plan);
-void fused_prop_table(const bpm_plan_s* plan, int row, std::vector<float2>* out);
-// (P^frac - 1)/N per band in the fused FFT's output order (nx <= 4096): the
-// propagator increment of a stage of frac * dz
-void fused_prop_table_frac(const bpm_plan_s* plan, int row, double frac,
-                           std::vector<float2>* out);
+// (P^frac - 1)/N of `row` in FP64, [band][frequency k]: the propagator
+// increments of a step (frac = 1) or a stage of frac * dz, from which the
+// FP32 kernels' tables below are taken, each value rounded once
+void prop_increments(const bpm_plan_s* plan, int row, double frac,
+                     std::vector<std::complex<double>>* out);
+// in the fused FFT's output order (nx <= 4096; the split tables above that)
+void fused_prop_table(const bpm_plan_s* plan, const std::vector<std::complex<double>>& inc,
+                      std::vector<float2>* out);
+// in natural frequency order, [2][nx] (spread kernels)
+void natural_prop_table(const std::vector<std::complex<double>>& inc, float2* out);
 // 3D: (P(qx, qy) - 1)/(nx ny) per band, [band][y position][x position] in the
 // output orders of the radix-16 FFTs along y and x.
 void vol_prop_table(const bpm_plan_s* plan, int row, std::vector<float2>* out);
@@ -260,10 +271,8 @@ int launch_omega_to_t(const void* d_in, void* d_out, int nb, int nx,
 int fused_smem_bytes(int logn);
 int fused_rows_resident(int logn, int n_rows);
 // Tables of the split-band form with local length 2^logm (N = 2^logm P).
-void split_prop_table(const bpm_plan_s* plan, int row, int logm, std::vector<float2>* out);
-// the same tables for a propagation of frac * dz (a stage of Eq. split-op)
-void split_prop_table_frac(const bpm_plan_s* plan, int row, int logm, double frac,
-                           std::vector<float2>* out);
+void split_prop_table(const bpm_plan_s* plan, const std::vector<std::complex<double>>& inc,
+                      int logm, std::vector<float2>* out);
 int split_table_stride(const bpm_plan_s* plan, int logm);   // float2 per row
 // Layout codes of launch_fused_layout: -1 rule, 0 CTA per row, 1 2-CTA
 // cluster per row, 2 4-CTA cluster per row (N = 4096, half-band split, 8
@@ -309,6 +318,12 @@ int fr_split_table_order(int logn, std::vector<int>* pos);
 // position order below), nx per band table.
 int fr_cta_table_order(int logn, std::vector<int>* pos);
 int fused_rows_per_cta(int logn);
+// One row per cluster of 2^lc CTAs (spread_kernel.cuh): the march of n_rows
+// rows with splitting `split`; rows carry prop_nat.
+int launch_spread(int logn, int lc, int split, const RowDescF32* d_rows, int n_rows, int steps,
+                  const float4* d_tw, int* d_status, cudaStream_t st);
+int spread_capacity(int logn, int lc, int split);   // clusters resident at once
+int spread_choice(int logn, int rows, int split);   // lc of a launch, 0: not spread
 int fused_threads(int logn);
 
 }  // namespace bpm

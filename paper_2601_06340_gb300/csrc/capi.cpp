@@ -48,10 +48,12 @@ int dev_alloc(bpm_plan_s* plan, void** p, size_t bytes, const char* what) {
 
 void free_plan_memory(bpm_plan_s* plan) {
   vol_release(plan);
-  void** ptrs[] = {&plan->d_phasor, &plan->d_sep, &plan->d_prop, &plan->d_prop_split, &plan->d_tw, &plan->d_state,
+  void** ptrs[] = {&plan->d_phasor, &plan->d_sep, &plan->d_prop, &plan->d_prop_split,
+                   &plan->d_prop_nat, &plan->d_tw, &plan->d_state,
                    &plan->d_state2, &plan->d_rows, &plan->d_io, &plan->d_spec,
                    &plan->d_twy, reinterpret_cast<void**>(&plan->d_pwpart),
-                   &plan->d_stage_rows, &plan->d_stage_prop, &plan->d_stage_prop_split};
+                   &plan->d_stage_rows, &plan->d_stage_prop, &plan->d_stage_prop_split,
+                   &plan->d_stage_prop_nat};
   for (void** p : ptrs) {
     if (*p) cudaFree(*p);
     *p = nullptr;
@@ -75,6 +77,15 @@ int device_sm_count() {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return sms > 0 ? sms : 1;
+}
+
+// Whether a plan's rows march spread over clusters with some splitting (its
+// natural-order propagator tables exist exactly then).
+bool spread_rows(const bpm_plan_s* plan) {
+  if (plan->precision != BPM_FP32_FUSED || plan->ny > 1) return false;
+  for (int s : {BPM_SPLIT_FIRST_ORDER, BPM_SPLIT_VERLET, BPM_SPLIT_FOREST_RUTH})
+    if (spread_choice(plan->logn, plan->nb, s) > 0) return true;
+  return false;
 }
 
 }  // namespace
@@ -105,6 +116,9 @@ void fused_rows(bpm_plan_s* plan, float2* state, float2* rec, double* pw, int n_
       // [2 tables][split table in thread order] per row: t dz, (1 - 2t) dz
       d.prop_split = static_cast<const float2*>(plan->d_stage_prop_split) +
                      size_t(r) * 2 * split_table_stride(plan, plan->logn == kSplitLogN ? 12 : 11);
+    const bool fr = plan->split == BPM_SPLIT_FOREST_RUTH;   // [2 tables] per row
+    const void* nat = fr ? plan->d_stage_prop_nat : plan->d_prop_nat;
+    d.prop_nat = nat ? static_cast<const float2*>(nat) + size_t(r) * (fr ? 4 : 2) * n : nullptr;
     if (plan->sep_slices) {
       d.phasor = nullptr;
       d.srows = static_cast<const SepRow*>(plan->d_sep);
@@ -248,6 +262,7 @@ struct LaunchShape {
   int layout = -1;   // 1: cluster per row, 0: CTA per row, -1: the rule
   int chunk = 0;     // rotation chunk (CTA layout, more rows than resident)
   bool rotated = false;
+  int spread = 0;    // log2 of the CTAs per row (spread_kernel.cuh), 0: the layout's kernel
 };
 
 static std::mutex g_tune_mu;
@@ -308,8 +323,35 @@ static bool fr_staged(const bpm_plan_s* plan) {
   return fv && std::strcmp(fv, "staged") == 0;
 }
 
+// log2 of the CTAs that each row of a plan is spread over, 0 if not (any
+// BPM_FUSED_LAYOUT forces the other forms).
+static int spread_lc(const bpm_plan_s* plan) {
+  if (!plan->d_prop_nat || std::getenv("BPM_FUSED_LAYOUT")) return 0;
+  return spread_choice(plan->logn, plan->nb, plan->split);
+}
+
+static LaunchShape choose_layout(bpm_plan_s* plan, PlanAux* aux, const void* state, int n_begin,
+                                 int steps, cudaStream_t st);
+
 static LaunchShape choose_shape(bpm_plan_s* plan, PlanAux* aux, const void* state, int n_begin,
                                 int steps, cudaStream_t st) {
+  const int lc = spread_lc(plan);
+  if (lc == 0) return choose_layout(plan, aux, state, n_begin, steps, st);
+  // reported under the codes of the cluster layouts (bpm_launch_shape)
+  LaunchShape sh;
+  sh.spread = lc;
+  const int logn = plan->logn;
+  if (plan->split == BPM_SPLIT_VERLET)
+    sh.layout = logn >= 12 ? kLayoutSplit4Half : logn == 11 ? kLayoutCtaHalf : kLayoutClusterHalf;
+  else if (plan->split == BPM_SPLIT_FOREST_RUTH)
+    sh.layout = logn > kSplitLogN ? kLayoutStagedFR : logn >= 12 ? kLayoutSplit4FR : kLayoutClusterFR;
+  else if (logn == 12 || (logn < 12 && plan->nb > 1 && autotune_enabled()))
+    sh.layout = kLayoutSplit4;
+  return sh;
+}
+
+static LaunchShape choose_layout(bpm_plan_s* plan, PlanAux* aux, const void* state, int n_begin,
+                                 int steps, cudaStream_t st) {
   NvtxRange nvtx("bpm_launch_shape_search");
   LaunchShape rule;
   const int nb = plan->nb, logn = plan->logn;
@@ -551,7 +593,7 @@ static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, void* state, void* d_re
                              int(plane_of(plan)), steps, plan->dx_um * plan->dy_um, final_pw,
                              pw_stride, st);
   }
-  if (fr_staged(plan)) {
+  if (fr_staged(plan) && spread_lc(plan) == 0) {
     int rc = march_staged_fr(plan, aux, state, d_rec, d_pw, n_begin, n_end, captured, st);
     if (rc != BPM_OK) return rc;
     return launch_finish_f32(static_cast<const float2*>(state),
@@ -575,9 +617,12 @@ static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, void* state, void* d_re
       rc = upload(plan->d_rows, rows.data(), sizeof(RowDescF32) * rows.size(), st, captured,
                   "upload row descriptors");
       if (rc != BPM_OK) return rc;
-      rc = launch_fused_layout(plan->logn, static_cast<const RowDescF32*>(plan->d_rows), plan->nb,
-                               steps, static_cast<const float4*>(plan->d_tw), plan->d_status, st,
-                               sh.layout);
+      const RowDescF32* d_rows = static_cast<const RowDescF32*>(plan->d_rows);
+      const float4* tw = static_cast<const float4*>(plan->d_tw);
+      rc = sh.spread ? launch_spread(plan->logn, sh.spread, plan->split, d_rows, plan->nb, steps,
+                                     tw, plan->d_status, st)
+                     : launch_fused_layout(plan->logn, d_rows, plan->nb, steps, tw,
+                                           plan->d_status, st, sh.layout);
     } else {
       const int cap = sh.layout == kLayoutCtaHalf ? fused_half_capacity(plan->logn)
                       : sh.layout == kLayoutCtaFR ? fused_fr_capacity(plan->logn)
@@ -659,6 +704,7 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
                           4 * int(nb) <= device_sm_count();
   if (half_split)
     A(&pl->d_prop_split, nb * size_t(split_table_stride(pl, 11)) * cs, "split propagator tables");
+  if (spread_rows(pl)) A(&pl->d_prop_nat, nb * 2 * n * cs, "natural propagator tables");
   A(&pl->d_tw, size_t(pl->nx) * 16, "twiddles");
   if (vol) {
     A(&pl->d_twy, size_t(pl->ny) * 16, "twiddles along y");
@@ -722,16 +768,24 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
       std::vector<float4> tw;
       twiddle_table_f32(pl->nx, &tw);
       e = cudaMemcpyAsync(pl->d_tw, tw.data(), n * 16, cudaMemcpyHostToDevice, st);
+      std::vector<std::complex<double>> inc;
       for (int r = 0; r < pl->nb && e == cudaSuccess; ++r) {
         std::vector<float2> t;
-        fused_prop_table(pl, r, &t);
+        prop_increments(pl, r, 1.0, &inc);
+        fused_prop_table(pl, inc, &t);
         e = cudaMemcpyAsync(static_cast<float2*>(pl->d_prop) + size_t(r) * prop_stride(pl),
                             t.data(), t.size() * sizeof(float2), cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess && pl->d_prop_split) {
-          split_prop_table(pl, r, 11, &t);
+          split_prop_table(pl, inc, 11, &t);
           e = cudaMemcpyAsync(static_cast<float2*>(pl->d_prop_split) +
                                   size_t(r) * split_table_stride(pl, 11),
                               t.data(), t.size() * sizeof(float2), cudaMemcpyHostToDevice, st);
+        }
+        if (e == cudaSuccess && pl->d_prop_nat) {
+          t.resize(inc.size());
+          natural_prop_table(inc, t.data());
+          e = cudaMemcpyAsync(static_cast<float2*>(pl->d_prop_nat) + size_t(r) * 2 * n, t.data(),
+                              t.size() * sizeof(float2), cudaMemcpyHostToDevice, st);
         }
       }
     } else {
@@ -795,7 +849,8 @@ int bpm_set_splitting(bpm_plan_t plan, int32_t method) {
     return fail(BPM_ERR_INVALID, "unknown splitting method");
   if (method == BPM_SPLIT_FOREST_RUTH && plan->ny > 1)
     return fail(BPM_ERR_INVALID, "3D plans march first order or Verlet");
-  for (void** p : {&plan->d_stage_rows, &plan->d_stage_prop, &plan->d_stage_prop_split}) {
+  for (void** p : {&plan->d_stage_rows, &plan->d_stage_prop, &plan->d_stage_prop_split,
+                   &plan->d_stage_prop_nat}) {
     if (*p) cudaFree(*p);
     *p = nullptr;
   }
@@ -818,15 +873,18 @@ int bpm_set_splitting(bpm_plan_t plan, int32_t method) {
                      "splitting propagators");
       if (rc != BPM_OK) return rc;
       std::vector<float2> host(nb * 2 * ts);
+      std::vector<std::complex<double>> inc;
+      std::vector<float2> nat(plan->d_prop_nat ? nb * 4 * n : 0);
       for (size_t r = 0; r < nb; ++r)
         for (int k = 0; k < 2; ++k) {
           std::vector<float2> tab;
           float2* dst = host.data() + (r * 2 + k) * ts;
+          prop_increments(plan, int(r), stages[1 + k].first, &inc);
+          if (plan->d_prop_nat) natural_prop_table(inc, nat.data() + (r * 2 + k) * 2 * n);
+          fused_prop_table(plan, inc, &tab);
           if (plan->logn >= kSplitLogN) {
-            split_prop_table_frac(plan, int(r), 12, stages[1 + k].first, &tab);
             std::copy(tab.begin(), tab.end(), dst);
           } else {
-            fused_prop_table_frac(plan, int(r), stages[1 + k].first, &tab);
             for (size_t b = 0; b < 2; ++b)
               for (size_t i = 0; i < n; ++i) dst[b * n + i] = tab[b * n + size_t(cpos[i])];
           }
@@ -836,6 +894,15 @@ int bpm_set_splitting(bpm_plan_t plan, int32_t method) {
                                       host.size() * sizeof(float2), cudaMemcpyHostToDevice, st);
       if (e == cudaSuccess) e = cudaStreamSynchronize(st);
       if (e != cudaSuccess) return cuda_fail(e, "splitting tables");
+      if (plan->d_prop_nat) {
+        rc = dev_alloc(plan, &plan->d_stage_prop_nat, nat.size() * sizeof(float2),
+                       "splitting propagators (spread kernels)");
+        if (rc != BPM_OK) return rc;
+        e = cudaMemcpyAsync(plan->d_stage_prop_nat, nat.data(), nat.size() * sizeof(float2),
+                            cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return cuda_fail(e, "splitting tables");
+      }
       if (plan->d_prop_split || plan->logn == kSplitLogN) {
         // the split kernels' fused forms (nx = 4096 rows that get four SMs,
         // nx = 8192): the tables of the t dz and (1 - 2t) dz propagations,
@@ -853,7 +920,8 @@ int bpm_set_splitting(bpm_plan_t plan, int32_t method) {
         for (size_t r = 0; r < nb; ++r)
           for (int k = 0; k < 2; ++k) {
             std::vector<float2> tab;
-            split_prop_table_frac(plan, int(r), slog, stages[1 + k].first, &tab);
+            prop_increments(plan, int(r), stages[1 + k].first, &inc);
+            split_prop_table(plan, inc, slog, &tab);
             float2* dst = hh.data() + (r * 2 + k) * hs;
             for (size_t q = 0; q < 4; ++q)
               for (size_t i = 0; i < m; ++i) dst[q * m + i] = tab[q * m + size_t(pos[i])];

@@ -52,6 +52,13 @@ cd expm1_i(cd z) {
   return cd(em * std::cos(x) + cosm1, ey * std::sin(x));
 }
 
+// exp(i x) - 1 for real x without cancellation (the same value as above, with
+// the terms that are exactly 0 or 1 left out).
+cd expm1_i(double x) {
+  const double sh = std::sin(0.5 * x);
+  return cd(-2.0 * sh * sh, std::sin(x));
+}
+
 double fftfreq_q(int k, int n, double dxh) {
   int kk = (k < n / 2) ? k : k - n;
   return kTwoPi * (double(kk) * (1.0 / (double(n) * dxh)));
@@ -203,13 +210,8 @@ std::vector<int> fft_output_order(int logn) {
 //          size, so a single float would round the small ones far beyond
 //          their own size, and that error repeats every step; hi + lo keeps
 //          it at FP64 level.
-void split_prop_table(const bpm_plan_s* plan, int row, int logm, std::vector<float2>* out) {
-  split_prop_table_frac(plan, row, logm, 1.0, out);
-}
-
-void split_prop_table_frac(const bpm_plan_s* plan, int row, int logm, double frac,
-                           std::vector<float2>* out) {
-  const EnergyConsts& c = plan->ec[row];
+void split_prop_table(const bpm_plan_s* plan, const std::vector<cd>& inc, int logm,
+                      std::vector<float2>* out) {
   const int n = plan->nx, m = 1 << logm, parts = n / m;
   std::vector<int> local = fft_output_order(logm);
   out->assign(size_t(split_table_stride(plan, logm)), float2{0.f, 0.f});
@@ -220,12 +222,8 @@ void split_prop_table_frac(const bpm_plan_s* plan, int row, int logm, double fra
     w[r] = cd(cr, ci);
   }
   for (int band = 0; band < 2; ++band) {
-    int sign = band == 0 ? +1 : -1;
     for (int pos = 0; pos < m; ++pos) {
-      for (int r = 0; r < parts; ++r) {
-        double q = fftfreq_q(local[pos] + m * r, n, c.dxh);
-        dk[r] = expm1_i(cd(frac * c.dzh * delta_q(q, c.s, c.c, sign), 0.0)) * (1.0 / double(n));
-      }
+      for (int r = 0; r < parts; ++r) dk[r] = inc[size_t(band) * n + local[pos] + m * r];
       if (parts == 2) {
         for (int r = 0; r < 2; ++r)
           (*out)[(size_t(band) * 2 + r) * m + pos] =
@@ -255,43 +253,40 @@ int split_table_stride(const bpm_plan_s* plan, int logm) {
   return parts == 2 ? 2 * parts * (1 << logm) : 2 * parts * parts * (1 << logm) * 2;
 }
 
-void fused_prop_table(const bpm_plan_s* plan, int row, std::vector<float2>* out) {
+void prop_increments(const bpm_plan_s* plan, int row, double frac, std::vector<cd>* out) {
   const EnergyConsts& c = plan->ec[row];
-  int n = plan->nx;
-  if (plan->logn >= kSplitLogN) {   // N = 4096 P, P = 2 or 4
-    split_prop_table(plan, row, 12, out);
-    return;
-  }
-  std::vector<int> order = fft_output_order(plan->logn);
-  out->assign(2 * size_t(n), float2{0.f, 0.f});
-  double inv_n = 1.0 / double(n);
+  const int n = plan->nx;
+  out->resize(2 * size_t(n));
+  const double inv_n = 1.0 / double(n);
   for (int band = 0; band < 2; ++band) {
-    int sign = band == 0 ? +1 : -1;
-    for (int pos = 0; pos < n; ++pos) {
-      double q = fftfreq_q(order[pos], n, c.dxh);
-      double ph = c.dzh * delta_q(q, c.s, c.c, sign);
-      cd d = expm1_i(cd(ph, 0.0)) * inv_n;
-      (*out)[size_t(band) * n + pos] = float2{float(d.real()), float(d.imag())};
+    const int sign = band == 0 ? +1 : -1;
+    for (int k = 0; k < n; ++k) {
+      const double q = fftfreq_q(k, n, c.dxh);
+      (*out)[size_t(band) * n + k] =
+          expm1_i(frac * c.dzh * delta_q(q, c.s, c.c, sign)) * inv_n;
     }
   }
 }
 
-void fused_prop_table_frac(const bpm_plan_s* plan, int row, double frac,
-                           std::vector<float2>* out) {
-  const EnergyConsts& c = plan->ec[row];
+void fused_prop_table(const bpm_plan_s* plan, const std::vector<cd>& inc,
+                      std::vector<float2>* out) {
+  if (plan->logn >= kSplitLogN) {   // N = 4096 P, P = 2 or 4
+    split_prop_table(plan, inc, 12, out);
+    return;
+  }
   const int n = plan->nx;
   std::vector<int> order = fft_output_order(plan->logn);
-  out->assign(2 * size_t(n), float2{0.f, 0.f});
-  const double inv_n = 1.0 / double(n);
-  for (int band = 0; band < 2; ++band) {
-    const int sign = band == 0 ? +1 : -1;
+  out->resize(2 * size_t(n));
+  for (int band = 0; band < 2; ++band)
     for (int pos = 0; pos < n; ++pos) {
-      const double q = fftfreq_q(order[pos], n, c.dxh);
-      const double ph = frac * c.dzh * delta_q(q, c.s, c.c, sign);
-      const cd d = expm1_i(cd(ph, 0.0)) * inv_n;
+      const cd d = inc[size_t(band) * n + order[pos]];
       (*out)[size_t(band) * n + pos] = float2{float(d.real()), float(d.imag())};
     }
-  }
+}
+
+void natural_prop_table(const std::vector<cd>& inc, float2* out) {
+  for (size_t i = 0; i < inc.size(); ++i)
+    out[i] = float2{float(inc[i].real()), float(inc[i].imag())};
 }
 
 void vol_prop_table(const bpm_plan_s* plan, int row, std::vector<float2>* out) {
@@ -312,7 +307,7 @@ void vol_prop_table(const bpm_plan_s* plan, int row, std::vector<float2>* out) {
         const double t = qx + sign * c.s;
         const double root = std::sqrt(1.0 - t * t - qy * qy);
         const double delta = -(qx * (qx + sign * 2.0 * c.s) + qy * qy) / (root + c.c);
-        const cd d = expm1_i(cd(c.dzh * delta, 0.0)) * inv;
+        const cd d = expm1_i(c.dzh * delta) * inv;
         (*out)[(size_t(band) * ny + py) * nx + px] = float2{float(d.real()), float(d.imag())};
       }
     }
@@ -386,7 +381,28 @@ void twiddle_table_f32(int n, std::vector<float4>* out) {
   for (int m = 0; m < n; ++m) {
     double c, s;
     unit_root(m, n, &c, &s);
+    // of the floats next to (c, s), the pair whose modulus is nearest to one:
+    // a forward and an inverse pass multiply by W and its conjugate, so the
+    // modulus error is the one that repeats every step at the same modes
+    // (marches of 2000-6000 steps with the spread kernels' three twiddle
+    // passes: relative error 4.7e-6 -> 4.3e-6 at N = 8192, 3.6e-6 -> 3.1e-6 at
+    // 2048, no larger than the two-pass kernels')
     float ch = float(c), sh = float(s);
+    if ((8 * m) % n != 0) {
+      const float c0 = ch, s0 = sh;
+      double best = 1.0;
+      for (int i = -1; i <= 1; ++i)
+        for (int j = -1; j <= 1; ++j) {
+          const float ci = i == 0 ? c0 : std::nextafterf(c0, i * 2.f);
+          const float sj = j == 0 ? s0 : std::nextafterf(s0, j * 2.f);
+          const double err = std::fabs(double(ci) * ci + double(sj) * sj - 1.0);
+          if (err < best) {
+            best = err;
+            ch = ci;
+            sh = sj;
+          }
+        }
+    }
     float cl = float(c - double(ch)), sl = float(s - double(sh));
     (*out)[m] = float4{ch, sh, cl, sl};
   }

@@ -31,6 +31,7 @@
 #include <atomic>
 #include <chrono>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <condition_variable>
 #include <deque>
@@ -371,6 +372,24 @@ bool has_unscheduled(const Bucket& b) {
   return false;
 }
 
+// Whether a first-order FP32 request may march spread over a cluster.
+bool can_spread(const Request& r) {
+  return r.plan->split == BPM_SPLIT_FIRST_ORDER && r.plan->d_prop_nat != nullptr;
+}
+
+// SMs the active first-order FP32 rows would occupy spread over clusters.
+int spread_demand(Server& s) {
+  int d = 0;
+  for (auto& kv : s.buckets) {
+    int rows = 0;
+    for (auto& r : kv.second.members)
+      if (r->plan->precision == BPM_FP32_FUSED && can_spread(*r)) rows += r->plan->nb;
+    const int logn = rows > 0 ? kv.second.members.front()->plan->logn : 0;
+    d += rows << (logn <= 9 ? 2 : logn == 10 ? 3 : 4);
+  }
+  return d;
+}
+
 // SMs the active FP32 rows would occupy in their cluster layouts.
 int cluster_demand(Server& s) {
   int d = 0;
@@ -402,11 +421,27 @@ int launch_batch(Server& s, Bucket& b) {
     for (auto& r : b.members) tables = tables && r->plan->d_prop_split != nullptr;
     if (tables) layout = kLayoutSplit4;
   }
+  // First-order rows spread over clusters of up to 16 SMs: N >= 8192 always
+  // (a row's SM time is no more than on the split bands: 8192 24 against 22
+  // SM us per step at full load, 16384 71 against 78, and its latency half),
+  // smaller rows while the whole active set fits the GPU that way.
+  int spread = 0;
+  if (fp32 && !std::getenv("BPM_FUSED_LAYOUT") &&
+      (logn >= kSplitLogN || spread_demand(s) <= s.sm_count)) {
+    int rows = 0;
+    bool tables = true;
+    for (auto& r : b.members) {
+      rows += r->plan->nb;
+      tables = tables && (can_spread(*r) || r->plan->split != BPM_SPLIT_FIRST_ORDER);
+    }
+    if (tables) spread = spread_choice(logn, rows, BPM_SPLIT_FIRST_ORDER);
+  }
   size_t limit = b.members.size();
   if (fp32) {
     const bool cluster = layout < 0 && 2 * int(b.members.size()) <= s.sm_count;
-    limit = size_t(std::max(1, layout == kLayoutSplit4 ? fused_split4_capacity()
-                                                       : fused_launch_capacity(logn, cluster)));
+    limit = size_t(std::max(1, spread ? spread_capacity(logn, spread, BPM_SPLIT_FIRST_ORDER)
+                               : layout == kLayoutSplit4 ? fused_split4_capacity()
+                                                         : fused_launch_capacity(logn, cluster)));
     // rows of the splitting forms march on their own kernels (N <= 4096: one
     // CTA per row, on the half-step or the fourth-order form; N = 8192,
     // 16384: the split-band cluster forms); a batch holding any stays
@@ -492,8 +527,12 @@ int launch_batch(Server& s, Bucket& b) {
                       : split == BPM_SPLIT_FOREST_RUTH
                           ? (logn >= kSplitLogN ? kLayoutSplit4FR : kLayoutCtaFR)
                           : layout;
-      bt.err = launch_fused_layout(logn, b.d_rows + off, int(kv.second.size()), kv.first / 3,
-                                   s.d_tw[logn], bt.d_status, b.st, lay);
+      const int nr = int(kv.second.size()), steps = kv.first / 3;
+      bt.err = split == BPM_SPLIT_FIRST_ORDER && spread
+                   ? launch_spread(logn, spread, split, b.d_rows + off, nr, steps, s.d_tw[logn],
+                                   bt.d_status, b.st)
+                   : launch_fused_layout(logn, b.d_rows + off, nr, steps, s.d_tw[logn],
+                                         bt.d_status, b.st, lay);
       off += kv.second.size();
     }
   }
