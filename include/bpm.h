@@ -22,8 +22,10 @@
  *   state after step (i+1)*record_every.  Powers: [B][n_rec+1][2] doubles,
  *   P = dx * sum_j |psi_j|^2 per band, at each record and (last entry) for
  *   the returned state.
- * Precision: BPM_FP64_PLAIN marches complex128 with one kernel launch per
- *   FFT pass and per pointwise step; BPM_FP32_FUSED marches complex64 in a
+ * Precision: BPM_FP64_PLAIN marches complex128 -- nx >= 64 in one
+ *   cooperative launch over all rows, smaller nx with one kernel launch per
+ *   FFT pass and per pointwise step (the plain form, which
+ *   bpm_march_f64_noalloc takes at every nx); BPM_FP32_FUSED marches complex64 in a
  *   persistent kernel that keeps each row on chip for many steps, with every
  *   phase argument (propagator, strain phase, common phase) formed in FP64
  *   and rounded once.  FP32 plans return c64 records; FP64 plans c128.
@@ -320,7 +322,7 @@ int bpm_slice_form(bpm_plan_t plan, int32_t* form, int64_t* bytes);
  * runs where cudaMalloc is not allowed or not wanted (a host callback, a
  * process whose device memory is owned by another allocator or budget, an
  * embedding that must not grow its footprint after start-up).  It advances
- * caller-owned device buffers with the plain FP64 step of bpm_propagate
+ * caller-owned device buffers with the plain FP64 step
  * (one launch per Stockham pass, propagator and coupling) and calls no
  * cudaMalloc, cudaFree or allocating library routine: its working memory
  * (16 MiB ping-pong buffer, 8192-entry twiddle table, 1024 row descriptors)

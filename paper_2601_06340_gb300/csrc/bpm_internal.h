@@ -93,6 +93,30 @@ struct RowDescF64 {
   double gphase;
 };
 
+// One batch row of a fused FP64 launch (f64_kernel.cuh).
+struct F64Row {
+  double2* state;           // [2][N] raw envelopes (common phase removed)
+  const double2* prop;      // [2][N] (P(q)-1)/N in bit-reversed frequency order
+  const double2* prop2;     // Forest-Ruth: of the (1 - 2t) dz stage (prop: of t dz)
+  const double2* phasor;    // [nz][N] exp(i h u_x), (0,0) outside the crystal
+  double2* records;         // [n_rec][2][N] or null
+  double* powers;           // [n_rec+1][2] or null
+  double2 am1, b;           // the step's coupling (Forest-Ruth: the inner ones)
+  double2 am1h, bh;         // the outer couplings of a splitting form
+  double gphase, dx_um;
+};
+
+// A fused FP64 march: rows of one plan.
+struct F64March {
+  const F64Row* rows;
+  const double2* tw;        // f64_twiddles
+  unsigned* sync;           // grid-barrier counter, zero at launch
+  double* part;             // [nb][items][2] band-power parts of a record
+  double2* xbuf;            // [nb][2][N] exchange buffer
+  int* status;
+  int32_t nb, steps, split, n_begin, n_phase0, record_every;
+};
+
 // Per-plan runtime buffers of the march entry points (capi.cpp): the plan's
 // stream, the host-API record / power buffers, the common phase factors and
 // the rotated launch schedule.
@@ -153,7 +177,9 @@ struct bpm_plan_s {
   void* d_tw = nullptr;           // FP32: float4 [nx] hi/lo; FP64: double2 [nx]
   void* d_state = nullptr;        // [B][2][nx] c64 / c128
   void* d_state2 = nullptr;       // FP64 ping-pong buffer
-  void* d_rows = nullptr;         // RowDescF32[B] or RowDescF64[B]
+  void* d_rows = nullptr;         // RowDescF32[B], RowDescF64[B] or F64Row[B]
+  void* d_f64 = nullptr;          // fused FP64 marches: barrier counter, power parts,
+                                  // exchange buffer
   void* d_io = nullptr;           // [B][2][nx] c128 host-transfer staging
   int* d_status = nullptr;        // device status word
   void* d_spec = nullptr;         // 3D: [B][2][ny][nx] c64 x-spectra
@@ -253,6 +279,23 @@ int fused_cluster_sms(int logn);
 int vol_march(bpm_plan_s* plan, float2* state, float2* d_rec, double* d_pw, int n_begin,
               int n_end, cudaStream_t st);
 void vol_release(bpm_plan_s* plan);   // the captured march, if any
+// FP64 march of the plan's d_state (f64.cu): one launch for nx >= 64, else
+// plain_march's launch per pass; kStatus bits go to `status`.
+int march_f64(bpm_plan_s* plan, int n_begin, int n_end, int n_phase0, void* d_records,
+              double* d_powers, int* status, cudaStream_t st);
+bool f64_fused(const bpm_plan_s* plan);
+size_t f64_scratch_bytes(const bpm_plan_s* plan);   // fused plans only
+// (P - 1)/N per band in bit-reversed frequency order, [2][nx]; rev =
+// bit_reversal(logn)
+void f64_prop_table(const bpm_plan_s* plan, const std::vector<std::complex<double>>& inc,
+                    const std::vector<int>& rev, double2* out);
+std::vector<int> bit_reversal(int bits);
+// Twiddles of the fused FP64 march, each stage's 2^s values at [2^s, 2^(s+1)) in
+// the order of the threads: [N1] forward column stages, [N2] inverse row
+// stages, [N1 rows][N2] forward row stages, [N2 columns][N1] inverse column
+// stages.
+void f64_twiddles(const bpm_plan_s* plan, std::vector<double2>* out);
+size_t f64_twiddle_count(const bpm_plan_s* plan);
 int plain_march(bpm_plan_s* plan, int n_begin, int n_end, int n_phase0, void* d_records,
                 double* d_powers, cudaStream_t st);
 int launch_convert_in(const double2* src, float2* dst, size_t n, cudaStream_t st);

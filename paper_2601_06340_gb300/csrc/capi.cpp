@@ -50,7 +50,7 @@ void free_plan_memory(bpm_plan_s* plan) {
   vol_release(plan);
   void** ptrs[] = {&plan->d_phasor, &plan->d_sep, &plan->d_prop, &plan->d_prop_split,
                    &plan->d_prop_nat, &plan->d_tw, &plan->d_state,
-                   &plan->d_state2, &plan->d_rows, &plan->d_io, &plan->d_spec,
+                   &plan->d_state2, &plan->d_rows, &plan->d_f64, &plan->d_io, &plan->d_spec,
                    &plan->d_twy, reinterpret_cast<void**>(&plan->d_pwpart),
                    &plan->d_stage_rows, &plan->d_stage_prop, &plan->d_stage_prop_split,
                    &plan->d_stage_prop_nat};
@@ -636,7 +636,7 @@ static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, void* state, void* d_re
                              reinterpret_cast<const double*>(aux->d_g), plan->nb, plan->nx, steps,
                              plan->dx_um, final_pw, pw_stride, st);
   }
-  int rc = plain_march(plan, n_begin, n_end, n_begin, d_rec, d_pw, st);
+  int rc = march_f64(plan, n_begin, n_end, n_begin, d_rec, d_pw, plan->d_status, st);
   if (rc != BPM_OK) return rc;
   return launch_finish_f64(static_cast<const double2*>(plan->d_state), static_cast<double2*>(out),
                            reinterpret_cast<const double*>(aux->d_g), plan->nb, plan->nx, steps,
@@ -705,14 +705,17 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
   if (half_split)
     A(&pl->d_prop_split, nb * size_t(split_table_stride(pl, 11)) * cs, "split propagator tables");
   if (spread_rows(pl)) A(&pl->d_prop_nat, nb * 2 * n * cs, "natural propagator tables");
-  A(&pl->d_tw, size_t(pl->nx) * 16, "twiddles");
+  const bool f64 = f64_fused(pl);
+  A(&pl->d_tw, (f64 ? f64_twiddle_count(pl) : size_t(pl->nx)) * 16, "twiddles");
   if (vol) {
     A(&pl->d_twy, size_t(pl->ny) * 16, "twiddles along y");
     A(&pl->d_spec, nb * 2 * n * cs, "x-spectra");
   }
   A(&pl->d_state, nb * 2 * n * cs, "state");
-  if (pl->precision == BPM_FP64_PLAIN) A(&pl->d_state2, nb * 2 * n * cs, "state scratch");
-  A(&pl->d_rows, nb * std::max(sizeof(RowDescF32), sizeof(RowDescF64)), "row descriptors");
+  if (f64) A(&pl->d_f64, f64_scratch_bytes(pl), "FP64 exchange");
+  else if (pl->precision == BPM_FP64_PLAIN) A(&pl->d_state2, nb * 2 * n * cs, "state scratch");
+  A(&pl->d_rows, nb * std::max({sizeof(RowDescF32), sizeof(RowDescF64), sizeof(F64Row)}),
+    "row descriptors");
   A(&pl->d_io, nb * 2 * n * 16, "host staging");
   A(reinterpret_cast<void**>(&pl->d_status), sizeof(int), "status");
   PlanAux* aux = aux_of(pl);
@@ -787,6 +790,18 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
           e = cudaMemcpyAsync(static_cast<float2*>(pl->d_prop_nat) + size_t(r) * 2 * n, t.data(),
                               t.size() * sizeof(float2), cudaMemcpyHostToDevice, st);
         }
+      }
+    } else if (f64) {
+      std::vector<double2> tw, t(2 * n);
+      std::vector<std::complex<double>> inc;
+      const std::vector<int> rev = bit_reversal(pl->logn);
+      f64_twiddles(pl, &tw);
+      e = cudaMemcpyAsync(pl->d_tw, tw.data(), tw.size() * 16, cudaMemcpyHostToDevice, st);
+      for (int r = 0; r < pl->nb && e == cudaSuccess; ++r) {
+        prop_increments(pl, r, 1.0, &inc);
+        f64_prop_table(pl, inc, rev, t.data());
+        e = cudaMemcpyAsync(static_cast<double2*>(pl->d_prop) + size_t(r) * 2 * n, t.data(),
+                            t.size() * sizeof(double2), cudaMemcpyHostToDevice, st);
       }
     } else {
       std::vector<double2> tw;
@@ -941,6 +956,30 @@ int bpm_set_splitting(bpm_plan_t plan, int32_t method) {
   }
   plan->split = method;
   if (method == BPM_SPLIT_FIRST_ORDER) return BPM_OK;
+  if (f64_fused(plan)) {
+    // the fused march takes its couplings from the row descriptors;
+    // Forest-Ruth also needs the tables of its t dz and (1 - 2t) dz stages
+    if (method != BPM_SPLIT_FOREST_RUTH) return BPM_OK;
+    std::vector<double2> tab(2 * nb * 2 * n);
+    std::vector<std::complex<double>> inc;
+    const std::vector<int> rev = bit_reversal(plan->logn);
+    for (size_t k = 0; k < 2; ++k)
+      for (size_t r = 0; r < nb; ++r) {
+        prop_increments(plan, int(r), stages[1 + k].first, &inc);
+        f64_prop_table(plan, inc, rev, tab.data() + (k * nb + r) * 2 * n);
+      }
+    int rc = dev_alloc(plan, &plan->d_stage_prop, tab.size() * sizeof(double2),
+                       "splitting propagators");
+    if (rc != BPM_OK) {
+      plan->split = BPM_SPLIT_FIRST_ORDER;
+      return rc;
+    }
+    cudaStream_t ast = aux_of(plan)->stream;
+    cudaError_t e = cudaMemcpyAsync(plan->d_stage_prop, tab.data(), tab.size() * sizeof(double2),
+                                    cudaMemcpyHostToDevice, ast);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ast);
+    return e == cudaSuccess ? BPM_OK : cuda_fail(e, "splitting tables");
+  }
   // one table per distinct nonzero a_i
   std::vector<double> fracs;
   for (auto& st : stages)

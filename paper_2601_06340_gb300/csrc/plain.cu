@@ -5,8 +5,9 @@
 //   forward Stockham passes (radix 4, plus one radix-2 pass for odd log2 N)
 //   -> propagator multiply P(q)/N (natural order) -> inverse passes
 //   -> real-space coupling with the strain phasor and mask -> [record].
-// It is the FP64 reference form on the GPU and the baseline the fused FP32
-// kernel is measured against.
+// It is the FP64 reference form on the GPU and the baseline the fused kernels
+// are measured against; FP64 plans of nx >= 64 march in one launch
+// (f64_kernel.cuh), smaller ones and the allocation-free entry point here.
 #include <mutex>
 #include <string>
 #include <vector>

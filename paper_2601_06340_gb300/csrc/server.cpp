@@ -474,7 +474,7 @@ int launch_batch(Server& s, Bucket& b) {
     bt.items.push_back({r, steps});
     r->n_sched += steps;
     if (!fp32) {
-      bt.err = plain_march(p, n0, n0 + steps, 0, r->d_rec, r->d_pow, b.st);
+      bt.err = march_f64(p, n0, n0 + steps, 0, r->d_rec, r->d_pow, bt.d_status, b.st);
       if (bt.err != BPM_OK) break;
       continue;
     }
