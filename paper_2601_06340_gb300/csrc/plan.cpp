@@ -215,11 +215,11 @@ void split_prop_table(const bpm_plan_s* plan, const std::vector<cd>& inc, int lo
   const int n = plan->nx, m = 1 << logm, parts = n / m;
   std::vector<int> local = fft_output_order(logm);
   out->assign(size_t(split_table_stride(plan, logm)), float2{0.f, 0.f});
-  std::vector<cd> dk(parts), w(parts);
-  for (int r = 0; r < parts; ++r) {
+  std::vector<cd> dk(parts), root(parts == 2 ? 0 : n);   // root[m] = W_N^m
+  for (int m = 0; m < int(root.size()); ++m) {
     double cr, ci;
-    unit_root(r, parts, &cr, &ci);
-    w[r] = cd(cr, ci);
+    unit_root(m, n, &cr, &ci);
+    root[m] = cd(cr, ci);
   }
   for (int band = 0; band < 2; ++band) {
     for (int pos = 0; pos < m; ++pos) {
@@ -232,12 +232,10 @@ void split_prop_table(const bpm_plan_s* plan, const std::vector<cd>& inc, int lo
       }
       for (int dl = 0; dl < parts; ++dl) {
         cd e(0.0, 0.0);
-        for (int r = 0; r < parts; ++r) e += w[(dl * r) % parts] * dk[r];
+        for (int r = 0; r < parts; ++r) e += root[((dl * r) % parts) * m] * dk[r];
         for (int h = 0; h < parts; ++h) {
           const int sh = h + dl < parts ? dl : dl - parts;     // h' - h
-          double wr, wi;
-          unit_root(((sh * local[pos]) % n + n) % n, n, &wr, &wi);   // W_N^{sh k}
-          const cd f = e * cd(wr, wi);
+          const cd f = e * root[((sh * local[pos]) % n + n) % n];   // W_N^{sh k}
           const float fr = float(f.real()), fi = float(f.imag());
           const size_t at = 2 * (((size_t(band) * parts + h) * parts + dl) * m + pos);
           (*out)[at] = float2{fr, fi};
@@ -378,7 +376,20 @@ static void unit_root(int m, int n, double* cr, double* ci) {
 
 void twiddle_table_f32(int n, std::vector<float4>* out) {
   out->resize(n);
-  for (int m = 0; m < n; ++m) {
+  auto put = [&](int m, double c, double s, float ch, float sh) {
+    (*out)[m] = float4{ch, sh, float(c - double(ch)), float(s - double(sh))};
+  };
+  if (n < 8) {
+    for (int m = 0; m < n; ++m) {
+      double c, s;
+      unit_root(m, n, &c, &s);
+      put(m, c, s, float(c), float(s));
+    }
+    return;
+  }
+  // the first octant, exp(-i a) with a = 2 pi m / n <= pi / 4, and its mirror
+  // images
+  for (int m = 0; m <= n / 8; ++m) {
     double c, s;
     unit_root(m, n, &c, &s);
     // of the floats next to (c, s), the pair whose modulus is nearest to one:
@@ -386,9 +397,9 @@ void twiddle_table_f32(int n, std::vector<float4>* out) {
     // modulus error is the one that repeats every step at the same modes
     // (marches of 2000-6000 steps with the spread kernels' three twiddle
     // passes: relative error 4.7e-6 -> 4.3e-6 at N = 8192, 3.6e-6 -> 3.1e-6 at
-    // 2048, no larger than the two-pass kernels')
+    // 2048, no larger than the two-pass kernels)
     float ch = float(c), sh = float(s);
-    if ((8 * m) % n != 0) {
+    if (m != 0 && m != n / 8) {
       const float c0 = ch, s0 = sh;
       double best = 1.0;
       for (int i = -1; i <= 1; ++i)
@@ -403,8 +414,20 @@ void twiddle_table_f32(int n, std::vector<float4>* out) {
           }
         }
     }
-    float cl = float(c - double(ch)), sl = float(s - double(sh));
-    (*out)[m] = float4{ch, sh, cl, sl};
+    const int q = n / 4;
+    put(m, c, s, ch, sh);                              // (c, s), s <= 0
+    put(q - m, -s, -c, -sh, -ch);
+    put(q + m, s, -c, sh, -ch);
+    put(2 * q - m, -c, s, -ch, sh);
+    if (m == 0) {
+      put(2 * q, -c, -s, -ch, -sh);
+      put(3 * q, -s, c, -sh, ch);
+      continue;
+    }
+    put(2 * q + m, -c, -s, -ch, -sh);
+    put(3 * q - m, s, c, sh, ch);
+    put(3 * q + m, -s, c, -sh, ch);
+    put(4 * q - m, c, -s, ch, -sh);
   }
 }
 
