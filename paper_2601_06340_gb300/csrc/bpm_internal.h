@@ -186,7 +186,7 @@ struct bpm_plan_s {
   void* d_twy = nullptr;          // 3D: float4 [ny] twiddles along y
   double* d_pwpart = nullptr;     // 3D: [B][n_rec][2][ny] line power sums
   size_t pwpart_bytes = 0;
-  void* vol_graph = nullptr;      // 3D: captured march (vol.cu)
+  unsigned* d_sync = nullptr;     // 3D: grid-barrier counter
   // operator splitting (FP64 plans): stages of one step
   int32_t split = BPM_SPLIT_FIRST_ORDER;
   int32_t n_stages = 0;
@@ -229,8 +229,8 @@ void fused_prop_table(const bpm_plan_s* plan, const std::vector<std::complex<dou
                       std::vector<float2>* out);
 // in natural frequency order, [2][nx] (spread kernels)
 void natural_prop_table(const std::vector<std::complex<double>>& inc, float2* out);
-// 3D: (P(qx, qy) - 1)/(nx ny) per band, [band][y position][x position] in the
-// output orders of the radix-16 FFTs along y and x.
+// 3D: (P(qx, qy) - 1)/(nx ny) in the order of the column phase's threads
+// (vol_kernel.cuh).
 void vol_prop_table(const bpm_plan_s* plan, int row, std::vector<float2>* out);
 int validate_problem3d(const bpm_problem* p, int ny, double dy_um, double y0_um,
                        std::string* why);
@@ -278,7 +278,6 @@ int fused_cluster_sms(int logn);
 // phase); records / powers as for the 2D fused path.
 int vol_march(bpm_plan_s* plan, float2* state, float2* d_rec, double* d_pw, int n_begin,
               int n_end, cudaStream_t st);
-void vol_release(bpm_plan_s* plan);   // the captured march, if any
 // FP64 march of the plan's d_state (f64.cu): one launch for nx >= 64, else
 // plain_march's launch per pass; kStatus bits go to `status`.
 int march_f64(bpm_plan_s* plan, int n_begin, int n_end, int n_phase0, void* d_records,

@@ -47,11 +47,11 @@ int dev_alloc(bpm_plan_s* plan, void** p, size_t bytes, const char* what) {
 }
 
 void free_plan_memory(bpm_plan_s* plan) {
-  vol_release(plan);
   void** ptrs[] = {&plan->d_phasor, &plan->d_sep, &plan->d_prop, &plan->d_prop_split,
                    &plan->d_prop_nat, &plan->d_tw, &plan->d_state,
                    &plan->d_state2, &plan->d_rows, &plan->d_f64, &plan->d_io, &plan->d_spec,
                    &plan->d_twy, reinterpret_cast<void**>(&plan->d_pwpart),
+                   reinterpret_cast<void**>(&plan->d_sync),
                    &plan->d_stage_rows, &plan->d_stage_prop, &plan->d_stage_prop_split,
                    &plan->d_stage_prop_nat};
   for (void** p : ptrs) {
@@ -710,6 +710,7 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
   if (vol) {
     A(&pl->d_twy, size_t(pl->ny) * 16, "twiddles along y");
     A(&pl->d_spec, nb * 2 * n * cs, "x-spectra");
+    A(reinterpret_cast<void**>(&pl->d_sync), sizeof(unsigned), "grid barrier");
   }
   A(&pl->d_state, nb * 2 * n * cs, "state");
   if (f64) A(&pl->d_f64, f64_scratch_bytes(pl), "FP64 exchange");

@@ -35,6 +35,7 @@
 #include <stdint.h>
 
 #include "bpm_internal.h"
+#include "grid_barrier.cuh"
 
 namespace bpm {
 
@@ -49,11 +50,6 @@ struct F64Cfg {
   static constexpr int ITEMS = N / T;                // per batch row and phase
   static_assert(KC >= 1 && KR >= 1, "an item holds both bands of a column, and a row");
 };
-
-// Poll limits of the grid barrier: inside the march (a poll takes about
-// 0.6 us, so about one second), and of the first one, which may have to wait
-// for other kernels to leave the SMs that this launch's last CTAs need.
-constexpr int kF64Polls = 1 << 21, kF64FirstPolls = 1 << 26;
 
 __device__ __forceinline__ double2 dmul(double2 a, double2 b) {
   return make_double2(fma(a.x, b.x, -(a.y * b.y)), fma(a.x, b.y, a.y * b.x));
@@ -125,14 +121,11 @@ __global__ void __launch_bounds__(F64Cfg<LOGN>::T) f64_march_kernel(const F64Mar
   __shared__ double red[T / 32 * 2];
   __shared__ double psum[2][ITEMS];
   __shared__ int s_dead;
+  GridBarrier grid(a.sync, &s_dead);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int n_items = a.nb * ITEMS;
   const bool half = a.split != BPM_SPLIT_FIRST_ORDER;
   const int stages = a.split == BPM_SPLIT_FOREST_RUTH ? 3 : 1;
-  bool dead = false;          // a wait expired: no more waits, finish the loop
-  int polls = kF64FirstPolls;
-  uint32_t target = 0;        // of the grid barrier's counter
-  if (t == 0) s_dead = 0;
 
   // ---- this thread's place in an item of either phase
   int x_row, x_band, x_col, x_i, k_row, k_band, k_pos, k_i;
@@ -177,26 +170,6 @@ __global__ void __launch_bounds__(F64Cfg<LOGN>::T) f64_march_kernel(const F64Mar
     return (size_t(k_row) * 2 + k_band) * N + size_t(k_pos) * N2 + k_i + p * (N2 / 2);
   };
   auto x_cell = [&](int p) { return (x_i + p * XT) * N2 + x_col; };
-
-  // Grid barrier: a counter that every CTA raises once (compared by its
-  // distance from the target, so it may wrap).  After an expired wait the
-  // CTA raises and waits no more, and the others' waits expire too.
-  auto grid_sync = [&] {
-    target += gridDim.x;
-    __syncthreads();
-    if (t == 0 && !dead) {
-      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.sync) : "memory");
-      uint32_t v = 0;
-      int n = 0;
-      do {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.sync) : "memory");
-      } while (int32_t(v - target) < 0 && ++n < polls);
-      if (int32_t(v - target) < 0) s_dead = 1;
-    }
-    __syncthreads();
-    if (s_dead) dead = true;
-    polls = kF64Polls;
-  };
 
   double2 v0, v1;          // the field at the item's cells
   double2 e0, e1, f0, f1;  // slices of step n and (half) n + 1
@@ -296,7 +269,7 @@ __global__ void __launch_bounds__(F64Cfg<LOGN>::T) f64_march_kernel(const F64Mar
     __stcg(a.xbuf + x_elem(1), v1);
   }
   k_place(first);
-  grid_sync();
+  grid.sync();
 
   for (int it = 0; it < a.steps; ++it) {
     const int n = n_begin + it;
@@ -320,7 +293,7 @@ __global__ void __launch_bounds__(F64Cfg<LOGN>::T) f64_march_kernel(const F64Mar
       if (sg == 0) due = -1;
       x_place(first);
       fetch(n, end && !last);
-      grid_sync();
+      grid.sync();
       // ---- phase X
       for (int item = first; item < n_items; item += gridDim.x) {
         if (item != first) {
@@ -357,13 +330,13 @@ __global__ void __launch_bounds__(F64Cfg<LOGN>::T) f64_march_kernel(const F64Mar
       }
       k_place(first);
       if (rec && end && pow_on) due = slot;
-      if (!(last && end) || due >= 0) grid_sync();
+      if (!(last && end) || due >= 0) grid.sync();
     }
   }
   if (due >= 0)
     for (int item = blockIdx.x; item < n_items; item += gridDim.x)
       if (item % ITEMS == 0) sum_power(item / ITEMS, due);
-  if (dead) atomicOr(a.status, kStatusWaitTimeout);
+  if (grid.dead && t == 0) atomicOr(a.status, kStatusWaitTimeout);
 }
 
 }  // namespace bpm

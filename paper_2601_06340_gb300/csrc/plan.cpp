@@ -287,26 +287,49 @@ void natural_prop_table(const std::vector<cd>& inc, float2* out) {
     out[i] = float2{float(inc[i].real()), float(inc[i].imag())};
 }
 
+// Frequency of value j of thread t, at index j T + t (T = n/8 threads), of the
+// 3D march's transforms: radix-8 passes and one of the power of two that is
+// left, the last pass's group i of thread t being t + i T.
+static std::vector<int> vol_order(int logn) {
+  const int n = 1 << logn, T = n / 8, np = (logn + 2) / 3, rl = 1 << (logn - 3 * (np - 1));
+  std::vector<int> out(n);
+  for (int j = 0; j < 8; ++j)
+    for (int t = 0; t < T; ++t) {
+      int rem = (t + (j / rl) * T) * rl + j % rl, freq = 0, mult = 1, len = n;
+      for (int p = 0; p < np; ++p) {
+        const int r = p < np - 1 ? 8 : rl, stride = len / r;
+        freq += (rem / stride) * mult;
+        rem %= stride;
+        mult *= r;
+        len = stride;
+      }
+      out[j * T + t] = freq;
+    }
+  return out;
+}
+
 void vol_prop_table(const bpm_plan_s* plan, int row, std::vector<float2>* out) {
   // delta_+-(qx, qy) = sqrt(1 - (qx +- s)^2 - qy^2) - cos(alpha)
   //                  = -(qx (qx +- 2 s) + qy^2) / (sqrt(...) + cos(alpha))
   const EnergyConsts& c = plan->ec[row];
-  const int nx = plan->nx, ny = plan->ny;
+  const int nx = plan->nx, ny = plan->ny, ty = ny / 8;
   const double dyh = c.k_um * plan->dy_um;
-  std::vector<int> ox = fft_output_order(plan->logn), oy = fft_output_order(plan->logny);
+  const std::vector<int> ox = vol_order(plan->logn), oy = vol_order(plan->logny);
   const double inv = 1.0 / (double(nx) * double(ny));
-  out->assign(2 * size_t(nx) * ny, float2{0.f, 0.f});
+  out->resize(2 * size_t(nx) * ny);
+  // [band][tile of 4 columns][j][column, t]: what thread (column, t) reads
   for (int band = 0; band < 2; ++band) {
     const double sign = band == 0 ? 1.0 : -1.0;
-    for (int py = 0; py < ny; ++py) {
-      const double qy = fftfreq_q(oy[py], ny, dyh);
-      for (int px = 0; px < nx; ++px) {
-        const double qx = fftfreq_q(ox[px], nx, c.dxh);
-        const double t = qx + sign * c.s;
+    for (int x = 0; x < nx; ++x) {
+      const double qx = fftfreq_q(ox[x], nx, c.dxh);
+      const double t = qx + sign * c.s;
+      float2* col = out->data() + (size_t(band) * (nx / 4) + x / 4) * 4 * ny + (x % 4) * ty;
+      for (int i = 0; i < ny; ++i) {
+        const double qy = fftfreq_q(oy[i], ny, dyh);
         const double root = std::sqrt(1.0 - t * t - qy * qy);
         const double delta = -(qx * (qx + sign * 2.0 * c.s) + qy * qy) / (root + c.c);
         const cd d = expm1_i(c.dzh * delta) * inv;
-        (*out)[(size_t(band) * ny + py) * nx + px] = float2{float(d.real()), float(d.imag())};
+        col[size_t(i / ty) * 4 * ty + i % ty] = float2{float(d.real()), float(d.imag())};
       }
     }
   }

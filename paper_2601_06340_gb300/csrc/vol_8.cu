@@ -1,0 +1,2 @@
+#include "vol_launch.cuh"
+BPM_INSTANTIATE_VOL(8)
