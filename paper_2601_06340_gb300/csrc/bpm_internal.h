@@ -187,6 +187,7 @@ struct bpm_plan_s {
   double* d_pwpart = nullptr;     // 3D: [B][n_rec][2][ny] line power sums
   size_t pwpart_bytes = 0;
   unsigned* d_sync = nullptr;     // 3D: grid-barrier counter
+  void* d_finish = nullptr;       // launch_finish scratch
   // operator splitting (FP64 plans): stages of one step
   int32_t split = BPM_SPLIT_FIRST_ORDER;
   int32_t n_stages = 0;
@@ -301,13 +302,15 @@ int launch_convert_in(const double2* src, float2* dst, size_t n, cudaStream_t st
 // Upload `bytes` of host memory to `dst` through kernel parameters (used
 // while the stream is being captured into a graph).
 int upload_by_params(void* dst, const void* src, size_t bytes, cudaStream_t st);
+// out = state * g per row and, if final_powers, the lines' powers; scratch of
+// finish_scratch_bytes, zero at its first use.
 int launch_finish_f32(const float2* state, double2* out_c128, float2* out_c64,
-                      const double* gphase, int n_rows, int nx, int steps,
-                      double dx, double* final_powers, int power_stride,
+                      const double* gphase, int n_rows, int nx, double dx, double* final_powers,
+                      int power_stride, void* scratch, cudaStream_t st);
+int launch_finish_f64(const double2* state, double2* out, const double* gphase, int n_rows,
+                      int nx, double dx, double* final_powers, int power_stride, void* scratch,
                       cudaStream_t st);
-int launch_finish_f64(const double2* state, double2* out, const double* gphase,
-                      int n_rows, int nx, int steps, double dx,
-                      double* final_powers, int power_stride, cudaStream_t st);
+size_t finish_scratch_bytes(int n_rows, int nx);
 int launch_omega_to_t(const void* d_in, void* d_out, int nb, int nx,
                       int precision, cudaStream_t st);
 int fused_smem_bytes(int logn);

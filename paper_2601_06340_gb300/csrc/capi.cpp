@@ -49,7 +49,7 @@ int dev_alloc(bpm_plan_s* plan, void** p, size_t bytes, const char* what) {
 void free_plan_memory(bpm_plan_s* plan) {
   void** ptrs[] = {&plan->d_phasor, &plan->d_sep, &plan->d_prop, &plan->d_prop_split,
                    &plan->d_prop_nat, &plan->d_tw, &plan->d_state,
-                   &plan->d_state2, &plan->d_rows, &plan->d_f64, &plan->d_io, &plan->d_spec,
+                   &plan->d_state2, &plan->d_rows, &plan->d_f64, &plan->d_finish, &plan->d_io, &plan->d_spec,
                    &plan->d_twy, reinterpret_cast<void**>(&plan->d_pwpart),
                    reinterpret_cast<void**>(&plan->d_sync),
                    &plan->d_stage_rows, &plan->d_stage_prop, &plan->d_stage_prop_split,
@@ -590,8 +590,8 @@ static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, void* state, void* d_re
                              out_c128 ? static_cast<double2*>(out) : nullptr,
                              out_c128 ? nullptr : static_cast<float2*>(out),
                              reinterpret_cast<const double*>(aux->d_g), plan->nb,
-                             int(plane_of(plan)), steps, plan->dx_um * plan->dy_um, final_pw,
-                             pw_stride, st);
+                             int(plane_of(plan)), plan->dx_um * plan->dy_um, final_pw,
+                             pw_stride, plan->d_finish, st);
   }
   if (fr_staged(plan) && spread_lc(plan) == 0) {
     int rc = march_staged_fr(plan, aux, state, d_rec, d_pw, n_begin, n_end, captured, st);
@@ -599,8 +599,8 @@ static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, void* state, void* d_re
     return launch_finish_f32(static_cast<const float2*>(state),
                              out_c128 ? static_cast<double2*>(out) : nullptr,
                              out_c128 ? nullptr : static_cast<float2*>(out),
-                             reinterpret_cast<const double*>(aux->d_g), plan->nb, plan->nx, steps,
-                             plan->dx_um, final_pw, pw_stride, st);
+                             reinterpret_cast<const double*>(aux->d_g), plan->nb, plan->nx,
+                             plan->dx_um, final_pw, pw_stride, plan->d_finish, st);
   }
   if (plan->precision == BPM_FP32_FUSED) {
     std::vector<RowDescF32> rows;
@@ -633,14 +633,14 @@ static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, void* state, void* d_re
     return launch_finish_f32(static_cast<const float2*>(state),
                              out_c128 ? static_cast<double2*>(out) : nullptr,
                              out_c128 ? nullptr : static_cast<float2*>(out),
-                             reinterpret_cast<const double*>(aux->d_g), plan->nb, plan->nx, steps,
-                             plan->dx_um, final_pw, pw_stride, st);
+                             reinterpret_cast<const double*>(aux->d_g), plan->nb, plan->nx,
+                             plan->dx_um, final_pw, pw_stride, plan->d_finish, st);
   }
   int rc = march_f64(plan, n_begin, n_end, n_begin, d_rec, d_pw, plan->d_status, st);
   if (rc != BPM_OK) return rc;
   return launch_finish_f64(static_cast<const double2*>(plan->d_state), static_cast<double2*>(out),
-                           reinterpret_cast<const double*>(aux->d_g), plan->nb, plan->nx, steps,
-                           plan->dx_um, final_pw, pw_stride, st);
+                           reinterpret_cast<const double*>(aux->d_g), plan->nb, plan->nx,
+                           plan->dx_um, final_pw, pw_stride, plan->d_finish, st);
 }
 
 }  // namespace bpm
@@ -717,6 +717,8 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
   else if (pl->precision == BPM_FP64_PLAIN) A(&pl->d_state2, nb * 2 * n * cs, "state scratch");
   A(&pl->d_rows, nb * std::max({sizeof(RowDescF32), sizeof(RowDescF64), sizeof(F64Row)}),
     "row descriptors");
+  const size_t fin_bytes = finish_scratch_bytes(pl->nb, int(n));
+  A(&pl->d_finish, fin_bytes, "finish scratch");
   A(&pl->d_io, nb * 2 * n * 16, "host staging");
   A(reinterpret_cast<void**>(&pl->d_status), sizeof(int), "status");
   PlanAux* aux = aux_of(pl);
@@ -823,6 +825,7 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
         e = cudaMemcpyAsync(pl->d_rows, rows.data(), rows.size() * sizeof(RowDescF64),
                             cudaMemcpyHostToDevice, st);
     }
+    if (e == cudaSuccess) e = cudaMemsetAsync(pl->d_finish, 0, fin_bytes, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(pl->d_status, 0, sizeof(int), st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) rc = cuda_fail(e, "plan upload");

@@ -16,32 +16,90 @@ __global__ void convert_in_kernel(const double2* __restrict__ src, float2* __res
     dst[i] = make_float2(float(src[i].x), float(src[i].y));
 }
 
-// One block per (row, band): out = state * g_row (FP64 product), power of
-// the line in FP64 (fixed summation order).
-template <typename TIn>
-__global__ void finish_kernel(const TIn* __restrict__ state, double2* __restrict__ out128,
-                              float2* __restrict__ out64, const double2* __restrict__ g,
-                              int nx, double dx, double* __restrict__ pw, int pw_stride) {
-  __shared__ double part[32];
-  const int row = blockIdx.x >> 1, band = blockIdx.x & 1;
-  const size_t base = (size_t(row) * 2 + band) * nx;
+// out = state * g_row (FP64 product) of one (row, band) line, a block of
+// kFinishThreads * PER points of it, and, if pw, the line's power in FP64: the
+// blocks' parts summed in a fixed order by the line's last block to finish.
+// The FP64 instructions bound it (64 clocks each for a warp, 19 per SM), so a
+// line runs on many blocks: one block of 256 threads per line took 425 us of
+// a 512 x 256 plane and 8 us of a 2048-point line, this form 6 and 2.
+constexpr int kFinishThreads = 128;
+
+__device__ __forceinline__ double block_sum(double s) {
+  __shared__ double part[kFinishThreads / 32];
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+  __syncthreads();
+  double tot = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < kFinishThreads / 32; ++w) tot += part[w];
+  return tot;    // thread 0's
+}
+
+template <typename TIn, int PER>
+__global__ void __launch_bounds__(kFinishThreads)
+    finish_kernel(const TIn* __restrict__ state, double2* __restrict__ out128,
+                  float2* __restrict__ out64, const double2* __restrict__ g, int nx, int blocks,
+                  double dx, double* __restrict__ pw, int pw_stride, double* __restrict__ part,
+                  unsigned* __restrict__ count) {
+  const int line = blockIdx.x / blocks, blk = blockIdx.x % blocks;
+  const int row = line >> 1, band = line & 1;
+  const size_t base = size_t(line) * nx;
   const double2 gr = g[row];
   double s = 0.0;
-  for (int j = threadIdx.x; j < nx; j += blockDim.x) {
-    const double vx = double(state[base + j].x), vy = double(state[base + j].y);
-    s += vx * vx + vy * vy;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    const int j = (blk * PER + i) * kFinishThreads + threadIdx.x;
+    if (j >= nx) break;
+    const TIn v = state[base + j];
+    const double vx = double(v.x), vy = double(v.y);
+    if (pw) s = fma(vx, vx, fma(vy, vy, s));
     const double ox = vx * gr.x - vy * gr.y, oy = vx * gr.y + vy * gr.x;
     if (out128) out128[base + j] = make_double2(ox, oy);
     if (out64) out64[base + j] = make_float2(float(ox), float(oy));
   }
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0 && pw) {
-    double tot = 0.0;
-    for (int w = 0; w < int(blockDim.x >> 5); ++w) tot += part[w];
-    pw[size_t(row) * pw_stride + band] = tot * dx;
+  if (!pw) return;
+  const double tot = block_sum(s);
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    part[size_t(line) * blocks + blk] = tot;
+    __threadfence();
+    last = atomicAdd(&count[line], 1u) == unsigned(blocks - 1);
   }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double sum = 0.0;
+  for (int k = threadIdx.x; k < blocks; k += kFinishThreads)
+    sum += __ldcg(&part[size_t(line) * blocks + k]);
+  sum = block_sum(sum);
+  if (threadIdx.x == 0) {
+    pw[size_t(row) * pw_stride + band] = sum * dx;
+    count[line] = 0;      // for the next march
+  }
+}
+
+int finish_per(int nx) { return nx <= 16384 ? 1 : 8; }
+int finish_blocks(int nx) {
+  const int points = kFinishThreads * finish_per(nx);
+  return (nx + points - 1) / points;
+}
+
+template <typename TIn>
+int launch_finish(const TIn* state, double2* out128, float2* out64, const double* g, int n_rows,
+                  int nx, double dx, double* pw, int pw_stride, void* scratch, cudaStream_t st) {
+  const int blocks = finish_blocks(nx), lines = 2 * n_rows;
+  double* part = static_cast<double*>(scratch);
+  unsigned* count = reinterpret_cast<unsigned*>(part + size_t(lines) * blocks);
+  const double2* g2 = reinterpret_cast<const double2*>(g);
+  const unsigned grid = unsigned(lines) * unsigned(blocks);
+  if (finish_per(nx) == 1)
+    finish_kernel<TIn, 1><<<grid, kFinishThreads, 0, st>>>(state, out128, out64, g2, nx, blocks, dx,
+                                                           pw, pw_stride, part, count);
+  else
+    finish_kernel<TIn, 8><<<grid, kFinishThreads, 0, st>>>(state, out128, out64, g2, nx, blocks, dx,
+                                                           pw, pw_stride, part, count);
+  cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? BPM_OK : cuda_fail(e, "finish");
 }
 
 // Energy -> time: for each (band, x) line, out[band][x][m] =
@@ -165,24 +223,22 @@ int launch_convert_in(const double2* src, float2* dst, size_t n, cudaStream_t st
   return e == cudaSuccess ? BPM_OK : cuda_fail(e, "convert input");
 }
 
+size_t finish_scratch_bytes(int n_rows, int nx) {
+  return size_t(2 * n_rows) * (size_t(finish_blocks(nx)) * sizeof(double) + sizeof(unsigned));
+}
+
 int launch_finish_f32(const float2* state, double2* out_c128, float2* out_c64,
-                      const double* g, int n_rows, int nx, int /*steps*/, double dx,
-                      double* final_powers, int power_stride, cudaStream_t st) {
-  finish_kernel<float2><<<2 * n_rows, 256, 0, st>>>(state, out_c128, out_c64,
-                                                    reinterpret_cast<const double2*>(g), nx, dx,
-                                                    final_powers, power_stride);
-  cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? BPM_OK : cuda_fail(e, "finish (fp32)");
+                      const double* g, int n_rows, int nx, double dx,
+                      double* final_powers, int power_stride, void* scratch, cudaStream_t st) {
+  return launch_finish(state, out_c128, out_c64, g, n_rows, nx, dx, final_powers, power_stride,
+                       scratch, st);
 }
 
 int launch_finish_f64(const double2* state, double2* out, const double* g, int n_rows, int nx,
-                      int /*steps*/, double dx, double* final_powers, int power_stride,
+                      double dx, double* final_powers, int power_stride, void* scratch,
                       cudaStream_t st) {
-  finish_kernel<double2><<<2 * n_rows, 256, 0, st>>>(state, out, nullptr,
-                                                     reinterpret_cast<const double2*>(g), nx, dx,
-                                                     final_powers, power_stride);
-  cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? BPM_OK : cuda_fail(e, "finish (fp64)");
+  return launch_finish(state, out, static_cast<float2*>(nullptr), g, n_rows, nx, dx, final_powers,
+                       power_stride, scratch, st);
 }
 
 int launch_omega_to_t(const void* d_in, void* d_out, int nb, int nx, int precision,

@@ -273,12 +273,12 @@ int retire_enqueue(Server& s, Request& r) {
   int rc;
   if (p->precision == BPM_FP32_FUSED)
     rc = launch_finish_f32(static_cast<const float2*>(r.d_state), r.d_out, nullptr,
-                           reinterpret_cast<const double*>(r.d_g), p->nb, p->nx, p->nz, p->dx_um,
-                           r.d_pow + 2 * p->n_rec, pw_stride, st);
+                           reinterpret_cast<const double*>(r.d_g), p->nb, p->nx, p->dx_um,
+                           r.d_pow + 2 * p->n_rec, pw_stride, p->d_finish, st);
   else
     rc = launch_finish_f64(static_cast<const double2*>(p->d_state), r.d_out,
-                           reinterpret_cast<const double*>(r.d_g), p->nb, p->nx, p->nz, p->dx_um,
-                           r.d_pow + 2 * p->n_rec, pw_stride, st);
+                           reinterpret_cast<const double*>(r.d_g), p->nb, p->nx, p->dx_um,
+                           r.d_pow + 2 * p->n_rec, pw_stride, p->d_finish, st);
   if (rc != BPM_OK) return rc;
   char* h = static_cast<char*>(r.h_stage);
   e = cudaMemcpyAsync(h, r.d_out, nb * 2 * n * 16, cudaMemcpyDeviceToHost, st);
