@@ -283,6 +283,12 @@ int vol_march(bpm_plan_s* plan, float2* state, float2* d_rec, double* d_pw, int 
 // plain_march's launch per pass; kStatus bits go to `status`.
 int march_f64(bpm_plan_s* plan, int n_begin, int n_end, int n_phase0, void* d_records,
               double* d_powers, int* status, cudaStream_t st);
+// The two halves of a fused one: its row descriptors, and the launch once
+// they are in the plan's d_rows.
+void f64_rows(const bpm_plan_s* plan, void* d_records, double* d_powers,
+              std::vector<F64Row>* out);
+int launch_f64(bpm_plan_s* plan, int n_begin, int n_end, int n_phase0, bool records, int* status,
+               cudaStream_t st);
 bool f64_fused(const bpm_plan_s* plan);
 size_t f64_scratch_bytes(const bpm_plan_s* plan);   // fused plans only
 // (P - 1)/N per band in bit-reversed frequency order, [2][nx]; rev =
@@ -302,6 +308,20 @@ int launch_convert_in(const double2* src, float2* dst, size_t n, cudaStream_t st
 // Upload `bytes` of host memory to `dst` through kernel parameters (used
 // while the stream is being captured into a graph).
 int upload_by_params(void* dst, const void* src, size_t bytes, cudaStream_t st);
+// A march's input field: n complex values at src, c64 or c128 (kC128ToC64:
+// rounded to c64).
+struct MarchInput {
+  enum Kind { kC64, kC128ToC64, kC128 } kind;
+  const void* src;
+  size_t n;
+};
+// Input to the state buffer `dst` (nothing to copy if it is already there) and
+// two pieces of host data (the second may be empty) to the device, in one
+// launch; both pieces together within stage_fits.  Sources and destinations
+// aligned to their types.
+int launch_stage(const MarchInput& in, void* dst, void* d_a, const void* a, size_t bytes_a,
+                 void* d_b, const void* b, size_t bytes_b, cudaStream_t st);
+bool stage_fits(size_t bytes_a, size_t bytes_b);
 // out = state * g per row and, if final_powers, the lines' powers; scratch of
 // finish_scratch_bytes, zero at its first use.
 int launch_finish_f32(const float2* state, double2* out_c128, float2* out_c64,

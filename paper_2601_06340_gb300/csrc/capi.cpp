@@ -568,79 +568,123 @@ static int march_staged_fr(bpm_plan_s* plan, PlanAux* aux, void* state, void* d_
   return rc;
 }
 
-// Enqueue the march of all rows on `st`.  state: the buffer holding the
-// state at n_begin (c64 for FP32, the plan's d_state for FP64); outputs as
-// documented for bpm_propagate_device.
-static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, void* state, void* d_rec, double* d_pw,
-                         int n_begin, int n_end, void* out, bool out_c128, cudaStream_t st) {
+// The input field to the state buffer by itself (a copy, or the conversion).
+static int copy_input(const MarchInput& in, void* state, cudaStream_t st) {
+  if (in.src == state) return BPM_OK;
+  if (in.kind == MarchInput::kC128ToC64)
+    return launch_convert_in(static_cast<const double2*>(in.src), static_cast<float2*>(state), in.n,
+                             st);
+  const size_t bytes = in.n * (in.kind == MarchInput::kC64 ? 8 : 16);
+  cudaError_t e = cudaMemcpyAsync(state, in.src, bytes, cudaMemcpyDeviceToDevice, st);
+  return e == cudaSuccess ? BPM_OK : cuda_fail(e, "copy input");
+}
+
+// The start of a march: the input to the state buffer, the phase factors and
+// the row descriptors (may be empty) to the device -- in one launch for few
+// rows, else a copy and two uploads.
+static int stage_march(bpm_plan_s* plan, PlanAux* aux, const MarchInput& in, void* state,
+                       const std::vector<double2>& g, const void* rows, size_t row_bytes,
+                       cudaStream_t st, bool captured) {
+  const size_t gb = g.size() * sizeof(double2), align = in.kind == MarchInput::kC64 ? 8 : 16;
+  // (a copy takes sources of any alignment)
+  if (stage_fits(gb, row_bytes) && reinterpret_cast<uintptr_t>(in.src) % align == 0)
+    return launch_stage(in, state, aux->d_g, g.data(), gb, plan->d_rows, rows, row_bytes, st);
+  int rc = copy_input(in, state, st);
+  if (rc == BPM_OK) rc = upload(aux->d_g, g.data(), gb, st, captured, "upload phase factors");
+  if (rc == BPM_OK && row_bytes)
+    rc = upload(plan->d_rows, rows, row_bytes, st, captured, "upload row descriptors");
+  return rc;
+}
+
+// Enqueue the march of all rows on `st`.  in: the field at n_begin; state: the
+// buffer that holds it during the march (c64 for FP32, the plan's d_state for
+// FP64); outputs as documented for bpm_propagate_device.
+static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, const MarchInput& in, void* state,
+                         void* d_rec, double* d_pw, int n_begin, int n_end, void* out,
+                         bool out_c128, cudaStream_t st) {
   const int steps = n_end - n_begin;
   const bool captured = capturing(st);
+  const bool fp32 = plan->precision == BPM_FP32_FUSED;
   std::vector<double2> g;
   phase_factors(plan, steps, &g);
-  int urc = upload(aux->d_g, g.data(), sizeof(double2) * plan->nb, st, captured,
-                   "upload phase factors");
-  if (urc != BPM_OK) return urc;
-  double* final_pw = d_pw ? d_pw + 2 * plan->n_rec : nullptr;
-  const int pw_stride = 2 * (plan->n_rec + 1);
+  auto finish = [&]() {
+    double* final_pw = d_pw ? d_pw + 2 * plan->n_rec : nullptr;
+    const int pw_stride = 2 * (plan->n_rec + 1);
+    const double* dg = reinterpret_cast<const double*>(aux->d_g);
+    const double area = plan->ny > 1 ? plan->dx_um * plan->dy_um : plan->dx_um;
+    const int n = int(plane_of(plan));
+    return fp32 ? launch_finish_f32(static_cast<const float2*>(state),
+                                    out_c128 ? static_cast<double2*>(out) : nullptr,
+                                    out_c128 ? nullptr : static_cast<float2*>(out), dg, plan->nb,
+                                    n, area, final_pw, pw_stride, plan->d_finish, st)
+                : launch_finish_f64(static_cast<const double2*>(plan->d_state),
+                                    static_cast<double2*>(out), dg, plan->nb, n, area, final_pw,
+                                    pw_stride, plan->d_finish, st);
+  };
+  int rc = BPM_OK;
+  if (!fp32) {
+    if (f64_fused(plan)) {
+      std::vector<F64Row> rows;
+      f64_rows(plan, d_rec, d_pw, &rows);
+      rc = stage_march(plan, aux, in, state, g, rows.data(), rows.size() * sizeof(F64Row), st,
+                       captured);
+      if (rc == BPM_OK)
+        rc = launch_f64(plan, n_begin, n_end, n_begin, d_rec || d_pw, plan->d_status, st);
+    } else {
+      rc = stage_march(plan, aux, in, state, g, nullptr, 0, st, captured);
+      if (rc == BPM_OK) rc = plain_march(plan, n_begin, n_end, n_begin, d_rec, d_pw, st);
+    }
+    return rc == BPM_OK ? finish() : rc;
+  }
   if (plan->ny > 1) {
-    int rc = vol_march(plan, static_cast<float2*>(state), static_cast<float2*>(d_rec), d_pw,
-                       n_begin, n_end, st);
-    if (rc != BPM_OK) return rc;
-    return launch_finish_f32(static_cast<const float2*>(state),
-                             out_c128 ? static_cast<double2*>(out) : nullptr,
-                             out_c128 ? nullptr : static_cast<float2*>(out),
-                             reinterpret_cast<const double*>(aux->d_g), plan->nb,
-                             int(plane_of(plan)), plan->dx_um * plan->dy_um, final_pw,
-                             pw_stride, plan->d_finish, st);
+    rc = stage_march(plan, aux, in, state, g, nullptr, 0, st, captured);
+    if (rc == BPM_OK)
+      rc = vol_march(plan, static_cast<float2*>(state), static_cast<float2*>(d_rec), d_pw,
+                     n_begin, n_end, st);
+    return rc == BPM_OK ? finish() : rc;
   }
   if (fr_staged(plan) && spread_lc(plan) == 0) {
-    int rc = march_staged_fr(plan, aux, state, d_rec, d_pw, n_begin, n_end, captured, st);
-    if (rc != BPM_OK) return rc;
-    return launch_finish_f32(static_cast<const float2*>(state),
-                             out_c128 ? static_cast<double2*>(out) : nullptr,
-                             out_c128 ? nullptr : static_cast<float2*>(out),
-                             reinterpret_cast<const double*>(aux->d_g), plan->nb, plan->nx,
-                             plan->dx_um, final_pw, pw_stride, plan->d_finish, st);
+    rc = stage_march(plan, aux, in, state, g, nullptr, 0, st, captured);
+    if (rc == BPM_OK)
+      rc = march_staged_fr(plan, aux, state, d_rec, d_pw, n_begin, n_end, captured, st);
+    return rc == BPM_OK ? finish() : rc;
   }
-  if (plan->precision == BPM_FP32_FUSED) {
-    std::vector<RowDescF32> rows;
-    fused_rows(plan, static_cast<float2*>(state), static_cast<float2*>(d_rec), d_pw, n_begin,
-               n_end, &rows);
-    const LaunchShape sh = choose_shape(plan, aux, state, n_begin, steps, st);
-    plan->shape_layout = sh.layout;
-    plan->shape_chunk =
-        sh.rotated ? std::min(steps, sh.chunk > 0 ? sh.chunk
-                                                  : std::max(std::min(steps, 64), steps / 24))
-                   : 0;
-    int rc = BPM_OK;
-    if (!sh.rotated) {
-      rc = upload(plan->d_rows, rows.data(), sizeof(RowDescF32) * rows.size(), st, captured,
-                  "upload row descriptors");
-      if (rc != BPM_OK) return rc;
-      const RowDescF32* d_rows = static_cast<const RowDescF32*>(plan->d_rows);
-      const float4* tw = static_cast<const float4*>(plan->d_tw);
-      rc = sh.spread ? launch_spread(plan->logn, sh.spread, plan->split, d_rows, plan->nb, steps,
-                                     tw, plan->d_status, st)
-                     : launch_fused_layout(plan->logn, d_rows, plan->nb, steps, tw,
-                                           plan->d_status, st, sh.layout);
-    } else {
-      const int cap = sh.layout == kLayoutCtaHalf ? fused_half_capacity(plan->logn)
-                      : sh.layout == kLayoutCtaFR ? fused_fr_capacity(plan->logn)
-                                                  : fused_launch_capacity(plan->logn, false);
-      rc = launch_rotated(plan, aux, rows, n_begin, steps, cap, st, sh.chunk, sh.layout);
-    }
+  std::vector<RowDescF32> rows;
+  fused_rows(plan, static_cast<float2*>(state), static_cast<float2*>(d_rec), d_pw, n_begin, n_end,
+             &rows);
+  const size_t row_bytes = sizeof(RowDescF32) * rows.size();
+  // the search for a batch's launch shape marches trials from the state
+  // buffer, so the input goes there first
+  MarchInput from = in;
+  if (spread_lc(plan) == 0 && plan->nb > 1) {
+    rc = copy_input(in, state, st);
     if (rc != BPM_OK) return rc;
-    return launch_finish_f32(static_cast<const float2*>(state),
-                             out_c128 ? static_cast<double2*>(out) : nullptr,
-                             out_c128 ? nullptr : static_cast<float2*>(out),
-                             reinterpret_cast<const double*>(aux->d_g), plan->nb, plan->nx,
-                             plan->dx_um, final_pw, pw_stride, plan->d_finish, st);
+    from.src = state;
+    from.kind = MarchInput::kC64;
   }
-  int rc = march_f64(plan, n_begin, n_end, n_begin, d_rec, d_pw, plan->d_status, st);
+  const LaunchShape sh = choose_shape(plan, aux, state, n_begin, steps, st);
+  plan->shape_layout = sh.layout;
+  plan->shape_chunk =
+      sh.rotated ? std::min(steps, sh.chunk > 0 ? sh.chunk
+                                                : std::max(std::min(steps, 64), steps / 24))
+                 : 0;
+  rc = stage_march(plan, aux, from, state, g, rows.data(), sh.rotated ? 0 : row_bytes, st,
+                   captured);
   if (rc != BPM_OK) return rc;
-  return launch_finish_f64(static_cast<const double2*>(plan->d_state), static_cast<double2*>(out),
-                           reinterpret_cast<const double*>(aux->d_g), plan->nb, plan->nx,
-                           plan->dx_um, final_pw, pw_stride, plan->d_finish, st);
+  if (!sh.rotated) {
+    const RowDescF32* d_rows = static_cast<const RowDescF32*>(plan->d_rows);
+    const float4* tw = static_cast<const float4*>(plan->d_tw);
+    rc = sh.spread ? launch_spread(plan->logn, sh.spread, plan->split, d_rows, plan->nb, steps,
+                                   tw, plan->d_status, st)
+                   : launch_fused_layout(plan->logn, d_rows, plan->nb, steps, tw, plan->d_status,
+                                         st, sh.layout);
+  } else {
+    const int cap = sh.layout == kLayoutCtaHalf ? fused_half_capacity(plan->logn)
+                    : sh.layout == kLayoutCtaFR ? fused_fr_capacity(plan->logn)
+                                                : fused_launch_capacity(plan->logn, false);
+    rc = launch_rotated(plan, aux, rows, n_begin, steps, cap, st, sh.chunk, sh.layout);
+  }
+  return rc == BPM_OK ? finish() : rc;
 }
 
 }  // namespace bpm
@@ -1168,16 +1212,10 @@ int bpm_propagate(bpm_plan_t plan, const double* psi_in, double* psi_out, void* 
   const size_t io_bytes = nb * 2 * n * 16;
   cudaError_t e = cudaMemcpyAsync(plan->d_io, psi_in, io_bytes, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_fail(e, "copy psi_in");
-  void* state = plan->d_state;
-  if (plan->precision == BPM_FP32_FUSED) {
-    rc = launch_convert_in(static_cast<const double2*>(plan->d_io), static_cast<float2*>(state),
-                           nb * 2 * n, st);
-  } else {
-    e = cudaMemcpyAsync(state, plan->d_io, io_bytes, cudaMemcpyDeviceToDevice, st);
-    rc = e == cudaSuccess ? BPM_OK : cuda_fail(e, "stage psi_in");
-  }
-  if (rc != BPM_OK) return rc;
-  rc = enqueue_march(plan, aux, state, want_rec ? aux->d_rec : nullptr,
+  const MarchInput in{plan->precision == BPM_FP32_FUSED ? MarchInput::kC128ToC64
+                                                        : MarchInput::kC128,
+                      plan->d_io, nb * 2 * n};
+  rc = enqueue_march(plan, aux, in, plan->d_state, want_rec ? aux->d_rec : nullptr,
                      want_pw ? aux->d_pow : nullptr, n_begin, n_end, plan->d_io, true, st);
   if (rc != BPM_OK) return rc;
   e = cudaMemcpyAsync(psi_out, plan->d_io, io_bytes, cudaMemcpyDeviceToHost, st);
@@ -1248,20 +1286,13 @@ int bpm_propagate_device(bpm_plan_t plan, const void* d_psi_in, void* d_psi_out,
       return fail(BPM_ERR_INVALID, "march the plan once outside the graph capture first");
   }
   if (plan->slices_dirty && (rc = prepare_slices(plan, aux->stream)) != BPM_OK) return rc;
-  const size_t bytes = size_t(plan->nb) * 2 * plane_of(plan) * csize(plan);
+  const size_t count = size_t(plan->nb) * 2 * plane_of(plan);
   void* rec = plan->n_rec > 0 ? d_records : nullptr;
-  if (plan->precision == BPM_FP32_FUSED) {
-    if (d_psi_out != d_psi_in) {
-      cudaError_t e = cudaMemcpyAsync(d_psi_out, d_psi_in, bytes, cudaMemcpyDeviceToDevice, st);
-      if (e != cudaSuccess) return cuda_fail(e, "copy input");
-    }
-    return enqueue_march(plan, aux, d_psi_out, rec, static_cast<double*>(d_powers), n_begin, n_end,
-                         d_psi_out, false, st);
-  }
-  cudaError_t e = cudaMemcpyAsync(plan->d_state, d_psi_in, bytes, cudaMemcpyDeviceToDevice, st);
-  if (e != cudaSuccess) return cuda_fail(e, "copy input");
-  return enqueue_march(plan, aux, plan->d_state, rec, static_cast<double*>(d_powers), n_begin,
-                       n_end, d_psi_out, true, st);
+  const bool fp32 = plan->precision == BPM_FP32_FUSED;
+  // FP32 marches in the output buffer, FP64 in the plan's
+  const MarchInput in{fp32 ? MarchInput::kC64 : MarchInput::kC128, d_psi_in, count};
+  return enqueue_march(plan, aux, in, fp32 ? d_psi_out : plan->d_state, rec,
+                       static_cast<double*>(d_powers), n_begin, n_end, d_psi_out, !fp32, st);
 }
 
 int bpm_device_status(bpm_plan_t plan, void* stream) {

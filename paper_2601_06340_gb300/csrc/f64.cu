@@ -121,15 +121,14 @@ size_t f64_scratch_bytes(const bpm_plan_s* plan) {
   return kF64SyncBytes + f64_part_bytes(plan) + size_t(plan->nb) * 2 * plan->nx * sizeof(double2);
 }
 
-int march_f64(bpm_plan_s* plan, int n_begin, int n_end, int n_phase0, void* d_records,
-              double* d_powers, int* status, cudaStream_t st) {
-  if (!f64_fused(plan)) return plain_march(plan, n_begin, n_end, n_phase0, d_records, d_powers, st);
+void f64_rows(const bpm_plan_s* plan, void* d_records, double* d_powers,
+              std::vector<F64Row>* out) {
   const size_t n = plan->nx, nb = plan->nb;
   const auto stages = split_stages(plan->split);
   const bool fr = plan->split == BPM_SPLIT_FOREST_RUTH;
-  std::vector<F64Row> rows(nb);
+  out->resize(nb);
   for (size_t r = 0; r < nb; ++r) {
-    F64Row& d = rows[r];
+    F64Row& d = (*out)[r];
     d.state = static_cast<double2*>(plan->d_state) + r * 2 * n;
     d.prop = static_cast<const double2*>(fr ? plan->d_stage_prop : plan->d_prop) + r * 2 * n;
     d.prop2 = fr ? d.prop + nb * 2 * n : nullptr;
@@ -153,10 +152,10 @@ int march_f64(bpm_plan_s* plan, int n_begin, int n_end, int n_phase0, void* d_re
     d.gphase = plan->ec[r].gphase;
     d.dx_um = plan->dx_um;
   }
-  // (pageable memory: the copy is staged before the call returns)
-  cudaError_t e = cudaMemcpyAsync(plan->d_rows, rows.data(), nb * sizeof(F64Row),
-                                  cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return cuda_fail(e, "upload row descriptors");
+}
+
+int launch_f64(bpm_plan_s* plan, int n_begin, int n_end, int n_phase0, bool records, int* status,
+               cudaStream_t st) {
   char* base = static_cast<char*>(plan->d_f64);
   F64March a{};
   a.rows = static_cast<const F64Row*>(plan->d_rows);
@@ -165,15 +164,28 @@ int march_f64(bpm_plan_s* plan, int n_begin, int n_end, int n_phase0, void* d_re
   a.part = reinterpret_cast<double*>(base + kF64SyncBytes);
   a.xbuf = reinterpret_cast<double2*>(base + kF64SyncBytes + f64_part_bytes(plan));
   a.status = status;
-  a.nb = int(nb);
+  a.nb = plan->nb;
   a.steps = n_end - n_begin;
   a.split = plan->split;
   a.n_begin = n_begin;
   a.n_phase0 = n_phase0;
-  a.record_every = (d_records || d_powers) ? plan->record_every : 0;
-  e = cudaMemsetAsync(base, 0, kF64SyncBytes, st);
+  a.record_every = records ? plan->record_every : 0;
+  cudaError_t e = cudaMemsetAsync(base, 0, kF64SyncBytes, st);
   if (e != cudaSuccess) return cuda_fail(e, "FP64 march");
   return with_size(plan->logn, [&](auto L) { return f64_launch<decltype(L)::value>(&a, st); });
+}
+
+
+int march_f64(bpm_plan_s* plan, int n_begin, int n_end, int n_phase0, void* d_records,
+              double* d_powers, int* status, cudaStream_t st) {
+  if (!f64_fused(plan)) return plain_march(plan, n_begin, n_end, n_phase0, d_records, d_powers, st);
+  std::vector<F64Row> rows;
+  f64_rows(plan, d_records, d_powers, &rows);
+  // (pageable memory: the copy is staged before the call returns)
+  cudaError_t e = cudaMemcpyAsync(plan->d_rows, rows.data(), rows.size() * sizeof(F64Row),
+                                  cudaMemcpyHostToDevice, st);
+  if (e != cudaSuccess) return cuda_fail(e, "upload row descriptors");
+  return launch_f64(plan, n_begin, n_end, n_phase0, d_records || d_powers, status, st);
 }
 
 }  // namespace bpm
