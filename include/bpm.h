@@ -152,9 +152,9 @@ int bpm_set_strain(bpm_plan_t plan, int32_t kind, const double* ux_um,
  * step, Verlet (half-step couplings on either side of the full-step
  * propagation) and Forest-Ruth (the leading coupling, then three
  * propagate-and-couple stages with the propagator increments of t dz and
- * (1 - 2t) dz, tabulated here once).  Rows of nx >= 512 march in one launch,
- * each spread over a cluster of 4 to 16 SMs while all rows of the plan run
- * at once that way (see bpm_launch_shape); more rows take one 4-CTA or 2-CTA
+ * (1 - 2t) dz, tabulated here once).  Rows march in one launch, one CTA per
+ * row or each spread over a cluster of 8 or 16 SMs (see bpm_launch_shape); where
+ * neither is the faster form they take one 4-CTA or 2-CTA
  * cluster per row while every row gets those SMs, else one CTA per row (nx
  * <= 4096) or one split-band cluster per row (nx >= 8192, Forest-Ruth for
  * nx = 8192 only).  BPM_FUSED_LAYOUT=staged (or any other value at nx =
@@ -350,10 +350,12 @@ int bpm_march_f64_noalloc(void* d_psi, int32_t nx, int32_t n_rows, const void* d
                           int32_t n_end, void* stream);
 
 /* Launch shape of the plan's last FP32 march (the fused kernels of the
- * step of Eq. fov10).  Rows of nx >= 512 are spread over clusters of 4, 8 or
- * 16 CTAs while that is the faster form (nx = 512 to about 250 rows, 1024
- * to 136, 2048 to 72, 4096 to 36, 8192 to 28, 16384 always but for 15 rows);
- * they report the code of their size's cluster form below.  *layout = 10
+ * step of Eq. fov10).  Rows of nx >= 64 march with 8 points per thread where
+ * that is the faster form: one CTA per row up to nx = 512 (any number of rows
+ * to nx = 128, 1000 rows of 256, 608 of 512) and for 137 to 304 rows of 1024,
+ * spread over clusters of 8 or 16 CTAs else (nx = 1024 to 136 rows, 2048 to
+ * 72, 4096 to 36, 8192 to 28, 16384 always but for 15 rows); they report the
+ * code below that their size and splitting had as single rows.  *layout = 10
  * the Forest-Ruth step on one cluster per row (512 <= nx <= 4096), 9 the
  * Forest-Ruth step on one cluster per row (nx = 4096 and 8192: 4-CTA
  * half-band split, split band), 8 the nx = 4096 half-band split with 16
@@ -365,9 +367,9 @@ int bpm_march_f64_noalloc(void* d_psi, int32_t nx, int32_t n_rows, const void* d
  * every nx <= 4096), 3 the Verlet step of nx = 2048 and on one CTA per row,
  * 2 one cluster per row (nx = 4096: spread, or two half-band parts per band
  * on four CTAs; smaller nx: spread batches), 1 one 2-CTA cluster per row,
- * 0 one CTA per row, -1 chosen by the fixed rule (spread, 2-CTA cluster while
- * every row gets two SMs, else one CTA per row).  BPM_FUSED_LAYOUT, set to any
- * value, keeps rows off the spread form.
+ * 0 one CTA per row, -1 chosen by the fixed rule (8 points per thread as
+ * above, 2-CTA cluster while every row gets two SMs, else one CTA per row).
+ * BPM_FUSED_LAYOUT, set to any value, keeps rows on the 16-point kernels.
  * *chunk = steps per launch of the rotation schedule (more rows than one
  * launch keeps resident), 0 for a single launch.  A batch march that is not
  * spread and has a choice of shapes (the layouts above for up to one row per

@@ -383,8 +383,10 @@ int fr_split_table_order(int logn, std::vector<int>* pos);
 // position order below), nx per band table.
 int fr_cta_table_order(int logn, std::vector<int>* pos);
 int fused_rows_per_cta(int logn);
-// One row per cluster of 2^lc CTAs (spread_kernel.cuh): the march of n_rows
-// rows with splitting `split`; rows carry prop_nat.
+// One row per cluster of 2^lc CTAs (spread_kernel.cuh), lc 2 to 4, or per CTA
+// (row_kernel.cuh), lc = kOneCta: the march of n_rows rows with splitting
+// `split`; rows carry prop_nat.
+constexpr int kOneCta = 1;
 int launch_spread(int logn, int lc, int split, const RowDescF32* d_rows, int n_rows, int steps,
                   const float4* d_tw, int* d_status, cudaStream_t st);
 int spread_capacity(int logn, int lc, int split);   // clusters resident at once

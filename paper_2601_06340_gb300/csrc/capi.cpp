@@ -342,11 +342,16 @@ static LaunchShape choose_shape(bpm_plan_s* plan, PlanAux* aux, const void* stat
   sh.spread = lc;
   const int logn = plan->logn;
   if (plan->split == BPM_SPLIT_VERLET)
-    sh.layout = logn >= 12 ? kLayoutSplit4Half : logn == 11 ? kLayoutCtaHalf : kLayoutClusterHalf;
+    sh.layout = logn >= 12               ? kLayoutSplit4Half
+                : logn == 11 || logn < 9 ? kLayoutCtaHalf
+                                         : kLayoutClusterHalf;
   else if (plan->split == BPM_SPLIT_FOREST_RUTH)
-    sh.layout = logn > kSplitLogN ? kLayoutStagedFR : logn >= 12 ? kLayoutSplit4FR : kLayoutClusterFR;
-  else if (logn == 12 || (logn < 12 && plan->nb > 1 && autotune_enabled()))
-    sh.layout = kLayoutSplit4;
+    sh.layout = logn > kSplitLogN ? kLayoutStagedFR
+                : logn >= 12      ? kLayoutSplit4FR
+                : logn >= 9       ? kLayoutClusterFR
+                                  : kLayoutCtaFR;
+  else if (logn == 12 || (logn >= 9 && logn < 12 && plan->nb > 1 && autotune_enabled()))
+    sh.layout = lc == kOneCta ? 0 : kLayoutSplit4;
   return sh;
 }
 

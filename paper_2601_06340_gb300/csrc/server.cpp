@@ -385,7 +385,7 @@ int spread_demand(Server& s) {
     for (auto& r : kv.second.members)
       if (r->plan->precision == BPM_FP32_FUSED && can_spread(*r)) rows += r->plan->nb;
     const int logn = rows > 0 ? kv.second.members.front()->plan->logn : 0;
-    d += rows << (logn <= 9 ? 2 : logn == 10 ? 3 : 4);
+    d += logn < 10 ? rows / 4 : rows << (logn == 10 ? 3 : 4);
   }
   return d;
 }
@@ -424,10 +424,12 @@ int launch_batch(Server& s, Bucket& b) {
   // First-order rows spread over clusters of up to 16 SMs: N >= 8192 always
   // (a row's SM time is no more than on the split bands: 8192 24 against 22
   // SM us per step at full load, 16384 71 against 78, and its latency half),
-  // smaller rows while the whole active set fits the GPU that way.
+  // N = 1024 to 4096 while the whole active set fits the GPU that way; N <= 512
+  // always one CTA of 8 points per thread, N = 1024 beyond that (2 rows per SM
+  // in 3.4 us either way, one in 2.0 against 3.4).
   int spread = 0;
-  if (fp32 && !std::getenv("BPM_FUSED_LAYOUT") &&
-      (logn >= kSplitLogN || spread_demand(s) <= s.sm_count)) {
+  if (fp32 && !std::getenv("BPM_FUSED_LAYOUT") && (logn <= 10 || logn >= kSplitLogN ||
+                                                   spread_demand(s) <= s.sm_count)) {
     int rows = 0;
     bool tables = true;
     for (auto& r : b.members) {
@@ -435,6 +437,8 @@ int launch_batch(Server& s, Bucket& b) {
       tables = tables && (can_spread(*r) || r->plan->split != BPM_SPLIT_FIRST_ORDER);
     }
     if (tables) spread = spread_choice(logn, rows, BPM_SPLIT_FIRST_ORDER);
+    if (spread && logn == 10 && spread_demand(s) > s.sm_count)
+      spread = rows <= spread_capacity(10, kOneCta, BPM_SPLIT_FIRST_ORDER) ? kOneCta : 0;
   }
   size_t limit = b.members.size();
   if (fp32) {

@@ -1,4 +1,4 @@
-// One row spread over a cluster of C = 4, 8 or 16 CTAs (an SM each): the
+// One row spread over a cluster of C = 8 or 16 CTAs (an SM each): the
 // march of rows while the GPU has SMs to spare for them.
 //
 // What bounds it.  A single row is a chain of z-steps, and a step a chain of
@@ -33,12 +33,11 @@
 // row thread (k1, band, r) starts with n2 = r + (N2/8) j.  With C = 8, point
 // j goes to CTA j, and the row thread of k1 = q, r = column has the sender's
 // own number t: it reads its j-th point at [j T + t], written by thread t of
-// CTA j.  With C = 16 (C = 4) one bit more selects the CTA (one bit of j is
-// left over): that bit is lane bit 4 ("hi"), q's top bit on the column side
-// and r's on the row side (the column's top bit and k1's).  So both
-// exchanges are the same permutation (spread_send), every warp receives
-// only from the warps of its own number and waits on its own barrier, all
-// reads are consecutive, and row transforms stay inside a warp.
+// CTA j.  With C = 16 one bit more selects the CTA: lane bit 4 ("hi"), q's top
+// bit on the column side and r's on the row side.  So both exchanges are the
+// same permutation, every warp receives only from the warps of its own number
+// and waits on its own barrier, all reads are consecutive, and row transforms
+// stay inside a warp.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -107,7 +106,7 @@ struct SpreadCfg {
   static constexpr int OFF_RED = OFF_PSLOT + 2 * C * 16;    // [WARPS][2] double
   static constexpr int OFF_RECPH = OFF_RED + WARPS * 16;    // [2] float2
   static constexpr int SMEM = OFF_RECPH + 16;
-  static_assert(C == 4 || C == 8 || C == 16, "cluster sizes with an exchange rule");
+  static_assert(C == 8 || C == 16, "cluster sizes with an exchange rule");
   static_assert(T >= 32 && T <= 256, "whole warps");
   static_assert(N1 <= 64 || (N1 == 128 && C == 16), "128-point columns pair across lane bit 4");
   static_assert(N2 <= 64 || (N2 == 128 && C >= 8), "128-point rows pair across a lane bit");
@@ -118,14 +117,14 @@ struct SpreadCfg {
 // Forward transform of L points held 8 per thread by threads of position q:
 // point j at index q + (L/8) j on entry, frequency q + (L/8) j on return.
 // addr(k, q') is the exchange buffer's slot of radix-8 output k of position
-// q'; w1[k - 1] = W_L^(q k); w2: W_16^((hi + 2 g) k), hi = bit 3 of q (L = 128).
-template <int L, typename AddrF, typename SyncF>
-__device__ __forceinline__ void spread_fwd(float2* v, float2* buf, int q, AddrF addr,
-                                           const float2* w1, const float2* w2, int xm,
-                                           SyncF sync) {
+// q'; w1(k) = W_L^(q k); w2: W_16^((hi + 2 g) k), hi = bit 3 of q (L = 128).
+template <int L, typename AddrF, typename TwF, typename SyncF>
+__device__ __forceinline__ void spread_fwd(float2* v, float2* buf, int q, AddrF addr, TwF w1,
+                                           const float2* w2, int xm, SyncF sync) {
   dft<8, false>(v);
+  if constexpr (L == 8) return;
 #pragma unroll
-  for (int k = 1; k < 8; ++k) v[k] = xmul(v[k], w1[k - 1]);
+  for (int k = 1; k < 8; ++k) v[k] = xmul(v[k], w1(k));
 #pragma unroll
   for (int k = 0; k < 8; ++k) buf[addr(k, q)] = v[k];
   sync();
@@ -175,10 +174,13 @@ __device__ __forceinline__ void spread_fwd(float2* v, float2* buf, int q, AddrF 
 }
 
 // The matching inverse (unnormalised): frequency q + (L/8) j on entry.
-template <int L, typename AddrF, typename SyncF>
-__device__ __forceinline__ void spread_inv(float2* v, float2* buf, int q, AddrF addr,
-                                           const float2* w1, const float2* w2, int xm,
-                                           SyncF sync) {
+template <int L, typename AddrF, typename TwF, typename SyncF>
+__device__ __forceinline__ void spread_inv(float2* v, float2* buf, int q, AddrF addr, TwF w1,
+                                           const float2* w2, int xm, SyncF sync) {
+  if constexpr (L == 8) {
+    dft<8, true>(v);
+    return;
+  }
   if constexpr (L <= 64) {
     constexpr int RL = L / 8, G = 8 / RL;
 #pragma unroll
@@ -222,7 +224,7 @@ __device__ __forceinline__ void spread_inv(float2* v, float2* buf, int q, AddrF 
 #pragma unroll
   for (int k = 0; k < 8; ++k) v[k] = buf[addr(k, q)];
 #pragma unroll
-  for (int k = 1; k < 8; ++k) v[k] = xmul(v[k], xconj(w1[k - 1]));
+  for (int k = 1; k < 8; ++k) v[k] = xmul(v[k], xconj(w1(k)));
   dft<8, true>(v);
 }
 
@@ -232,6 +234,52 @@ template <int LOGN>
 __device__ __forceinline__ int spread_cell(int x) {
   constexpr int PARTS = LOGN > 12 ? 1 << (LOGN - 12) : 1;
   return (x % PARTS) * ((1 << LOGN) / PARTS) + x / PARTS;
+}
+
+// One step's slice at a thread's 8 points: e[j] the phasor, (0, 0) outside the
+// crystal.  Separable rows hold the column phasors there for the launch and
+// take the inside mask m and the row phasor ph from the step's row head.
+struct Slice8 {
+  float2 e[8];
+  uint32_t m;
+  float2 ph;
+};
+
+// Slice of step n at cells x0 + j N/8.
+template <int LOGN>
+__device__ __forceinline__ void slice8_fetch(Slice8& s, const RowDescF32& d, int n, int x0,
+                                             bool sep) {
+  constexpr int N = 1 << LOGN;
+  if (sep) {
+    const float4 h = __ldg(reinterpret_cast<const float4*>(d.srows + n));
+    const SepHead sh{make_float2(h.x, h.y), __float_as_int(h.z), __float_as_int(h.w)};
+    s.m = sep_mask<0, LOGN - 3, 8>(sh, x0, 0);
+    s.ph = sh.ph;
+  } else {
+    const float2* p = d.phasor + size_t(n) * N;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s.e[j] = __ldg(&p[spread_cell<LOGN>(x0 + j * (N / 8))]);
+  }
+}
+
+// Couple the 8 points with coefficients (am1, b); the other band's values are
+// in lane ^ BM, sg = -1 in band 1.
+template <int BM>
+__device__ __forceinline__ void slice8_couple(float2* v, const Slice8& s, float2 am1, float2 b,
+                                              float sg, bool sep) {
+  uint32_t m = s.m;
+  if (sep) {          // the row phasor folded into b, conjugated for band 1
+    b = xmul(b, make_float2(s.ph.x, s.ph.y * sg));
+  } else {
+    m = 0u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      m |= ((s.e[j].x != 0.f) | (s.e[j].y != 0.f)) ? 1u << j : 0u;
+  }
+  const float2 bs = make_float2(b.x * sg, b.y * sg);
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    v[j] = xcouple(v[j], xshfl(v[j], BM), s.e[j], (m >> j) & 1u, am1, b, bs);
 }
 
 // SCH: the operator splitting as in fused2_kernel.cuh.
@@ -259,8 +307,8 @@ __global__ void __launch_bounds__((SpreadCfg<LOGN, LC>::T), 1)
   const int band = (tl % U) / CI, ci = tl % CI;
   const int q = (C == 16 ? hi * (S::Q / 2) : 0) + tl / U;       // column position
   const int r = (C == 16 ? hi * (S::RQ / 2) : 0) + ci;          // row position
-  const int n2 = c * (N2 / C) + (C == 4 ? hi * CI : 0) + ci;    // column
-  const int k1 = c * (N1 / C) + (C == 4 ? hi * S::Q : 0) + tl / U;   // row
+  const int n2 = c * (N2 / C) + ci;             // column
+  const int k1 = c * (N1 / C) + tl / U;         // row
   const int x0 = q * N2 + n2;                                   // cell of point j: x0 + j N/8
 
   float2* xf = reinterpret_cast<float2*>(smem + S::OFF_X0);
@@ -286,20 +334,16 @@ __global__ void __launch_bounds__((SpreadCfg<LOGN, LC>::T), 1)
   fence_mbar_init();
 
   bool timed_out = false;
-  // exchange: point j of this thread goes to slot `slot(j)` of CTA dst(j)
-  auto dst = [&](int j) { return uint32_t(C == 8 ? j : C == 16 ? 2 * j + hi : j >> 1); };
-  const int tb = t & ~16;
-  auto slot = [&](int j) {
-    return C == 8 ? c * T + t : C == 16 ? (c >> 1) * T + (tb | ((c & 1) << 4))
-                                        : (2 * c + hi) * T + (tb | ((j & 1) << 4));
-  };
+  // exchange: point j of this thread goes to slot `slot` of CTA dst(j)
+  auto dst = [&](int j) { return uint32_t(C == 8 ? j : 2 * j + hi); };
+  const int slot = C == 8 ? c * T + t : (c >> 1) * T + ((t & ~16) | ((c & 1) << 4));
   // remote addresses of point j's slot in the spectrum buffer and of the
   // warp's spectrum barrier; the increment's lie at fixed offsets from them
-  uint32_t rslot[8], rbar[C == 4 ? 4 : 8];
+  uint32_t rslot[8], rbar[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    rslot[j] = mapa_u32(smem_u32(fb + slot(j)), dst(j));
-    if (C != 4 || j % 2 == 0) rbar[C == 4 ? j / 2 : j] = mapa_u32(smem_u32(fbar), dst(j));
+    rslot[j] = mapa_u32(smem_u32(fb + slot), dst(j));
+    rbar[j] = mapa_u32(smem_u32(fbar), dst(j));
   }
   auto send = [&](const float2* v, auto inv) {
     constexpr bool INV = decltype(inv)::value;
@@ -310,11 +354,11 @@ __global__ void __launch_bounds__((SpreadCfg<LOGN, LC>::T), 1)
 #pragma unroll
     for (int j = 0; j < 8; ++j)
       st_async_v2<INV ? S::OFF_G - S::OFF_F : 0, INV ? S::OFF_GBAR - S::OFF_FBAR : 0>(
-          rslot[j], v[j], rbar[C == 4 ? j / 2 : j]);
+          rslot[j], v[j], rbar[j]);
   };
 
   // exchange slots inside the CTA (columns) and the warp (rows)
-  const int ucol = C == 4 ? hi * (T / 2) + tl % U : tl % U;
+  const int ucol = tl % U;
   auto col_addr = [&](int k, int pos) {
     if constexpr (C == 16)
       return k * S::P + (pos / (S::Q / 2)) * (T / 2) + (pos % (S::Q / 2)) * U + ucol;
@@ -323,7 +367,6 @@ __global__ void __launch_bounds__((SpreadCfg<LOGN, LC>::T), 1)
   const int rlane = C == 8 ? lane & ~(S::RQ - 1) : lane & 15 & ~(CI - 1);
   auto row_addr = [&](int k, int pos) {
     if constexpr (C == 16) return k * 33 + ((pos / CI) * 16 | rlane | (pos % CI));
-    else if constexpr (C == 4) return k * 33 + (hi * 16 | rlane | pos);
     else return k * 33 + (rlane | pos);
   };
   auto cta_sync = [] {
@@ -346,6 +389,8 @@ __global__ void __launch_bounds__((SpreadCfg<LOGN, LC>::T), 1)
   }
 #pragma unroll
   for (int j = 0; j < 8; ++j) wm[j] = root(n2 * (q + S::Q * j));
+  auto w_col = [&](int k) { return wc[k - 1]; };
+  auto w_row = [&](int k) { return wr[k - 1]; };
   // third-pass twiddles of 128-point transforms: positions h, h + 2 of 4
   float2 w2c[N1 == 128 ? 6 : 1], w2r[N2 == 128 ? 6 : 1];
 #pragma unroll
@@ -369,54 +414,16 @@ __global__ void __launch_bounds__((SpreadCfg<LOGN, LC>::T), 1)
 #pragma unroll
   for (int j = 0; j < 8; ++j) v[j] = d.state[band * N + x0 + j * (N / 8)];
 
-  // Slices: e[j] is the phasor of cell j, (0, 0) outside the crystal.
-  // Separable rows hold the column phasors there for the launch and take
-  // the inside mask m and the row phasor ph from the step's row head.
   const bool sep = d.srows != nullptr;
-  struct Slice {
-    float2 e[8];
-    uint32_t m;
-    float2 ph;
-  };
-  auto fetch = [&](Slice& s, int n) {
-    if (sep) {
-      const float4 h = __ldg(reinterpret_cast<const float4*>(d.srows + n));
-      const SepHead sh{make_float2(h.x, h.y), __float_as_int(h.z), __float_as_int(h.w)};
-      s.m = sep_mask<0, LOGN - 3, 8>(sh, x0, 0);
-      s.ph = sh.ph;
-    } else {
-      const float2* p = d.phasor + size_t(n) * N;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        s.e[j] = __ldg(&p[spread_cell<LOGN>(x0 + j * (N / 8))]);
-      }
-    }
-  };
-  Slice cur, nxt;
+  const float sg1 = band ? -1.f : 1.f;
+  Slice8 cur, nxt;
   if (sep)
 #pragma unroll
     for (int j = 0; j < 8; ++j)
       cur.e[j] = nxt.e[j] = __ldg(&d.scols[spread_cell<LOGN>(x0 + j * (N / 8))]);
-  // couple this thread's points on slice s with coefficients (am1, b)
-  const float sg1 = band ? -1.f : 1.f;
-  auto couple = [&](const Slice& s, float2 am1, float2 b) {
-    uint32_t m = s.m;
-    if (sep) {          // the row phasor folded into b, conjugated for band 1
-      float2 ph = s.ph;
-      ph.y *= sg1;
-      b = xmul(b, ph);
-    } else {
-      m = 0u;
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        m |= ((s.e[j].x != 0.f) | (s.e[j].y != 0.f)) ? 1u << j : 0u;
-    }
-    float2 bs = b;
-    bs.x *= sg1;
-    bs.y *= sg1;
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      v[j] = xcouple(v[j], xshfl(v[j], BM), s.e[j], (m >> j) & 1u, am1, b, bs);
+  auto fetch = [&](Slice8& s, int n) { slice8_fetch<LOGN>(s, d, n, x0, sep); };
+  auto couple = [&](const Slice8& s, float2 am1, float2 b) {
+    slice8_couple<BM>(v, s, am1, b, sg1, sep);
   };
 
   cluster.sync();   // every CTA's barriers initialised before any remote store
@@ -462,7 +469,7 @@ __global__ void __launch_bounds__((SpreadCfg<LOGN, LC>::T), 1)
       float2 org[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) org[j] = v[j];
-      spread_fwd<N1>(v, xf, q, col_addr, wc, w2c, 16, cta_sync);
+      spread_fwd<N1>(v, xf, q, col_addr, w_col, w2c, 16, cta_sync);
       if (part_due && sg == 0 && lead) {
         double p[2];
         cta_power(p);
@@ -481,19 +488,19 @@ __global__ void __launch_bounds__((SpreadCfg<LOGN, LC>::T), 1)
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = fb[j * T + t];
       __syncwarp();     // (the previous stage's reads of y)
-      spread_fwd<N2>(v, y, r, row_addr, wr, w2r, S::XM, warp_sync);
+      spread_fwd<N2>(v, y, r, row_addr, w_row, w2r, S::XM, warp_sync);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         if constexpr (TWO) v[j] = xmul(v[j], sg == 1 ? d1[j] : d0[j]);
         else v[j] = xmul(v[j], d0[j]);
       }
       __syncwarp();
-      spread_inv<N2>(v, y, r, row_addr, wr, w2r, S::XM, warp_sync);
+      spread_inv<N2>(v, y, r, row_addr, w_row, w2r, S::XM, warp_sync);
       send(v, BoolC<true>{});
       if (!timed_out && !mbar_wait_cluster(gbar, par)) timed_out = true;
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = xmul(gb[j * T + t], xconj(wm[j]));
-      spread_inv<N1>(v, xi, q, col_addr, wc, w2c, 16, cta_sync);
+      spread_inv<N1>(v, xi, q, col_addr, w_col, w2c, 16, cta_sync);
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = cadd(org[j], v[j]);
       if (part_due && sg == 0 && lead && c == 0) {

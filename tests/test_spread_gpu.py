@@ -1,4 +1,5 @@
-"""Rows spread over clusters of 4 to 16 CTAs (csrc/spread_kernel.cuh).
+"""Rows of 8 points per thread: spread over clusters of 8 or 16 CTAs
+(csrc/spread_kernel.cuh) or one row per CTA (csrc/row_kernel.cuh).
 
 Every size and cluster size of the form, on random two-band fields (every
 mode and cell carries weight) through a masked, strained crystal stored as a
@@ -39,7 +40,8 @@ def _workload(nx, rows):
 
 
 # (nx, rows): one row, then the counts at which the rule changes
-CASES = [(512, 1), (512, 101), (1024, 1), (1024, 77), (2048, 1), (2048, 7), (2048, 8),
+CASES = [(64, 1), (64, 33), (128, 1), (256, 5), (512, 1), (512, 101), (1024, 1), (1024, 77),
+         (1024, 151), (2048, 1), (2048, 7), (2048, 8),
          (4096, 1), (4096, 33), (8192, 1), (8192, 15), (8192, 17), (16384, 1), (16384, 8)]
 
 
