@@ -1,5 +1,5 @@
-// Input conversion, output finishing (common phase, final powers) and the
-// energy -> time synthesis of a batch of exit fields.
+// Input conversion, output finishing (common phase, final powers) and the start
+// of a march from host data.
 #include <algorithm>
 #include <cstring>
 
@@ -102,53 +102,6 @@ int launch_finish(const TIn* state, double2* out128, float2* out64, const double
   return e == cudaSuccess ? BPM_OK : cuda_fail(e, "finish");
 }
 
-// Energy -> time: for each (band, x) line, out[band][x][m] =
-// sum_j in[j][band][x] exp(-2 pi i j m / B) -- the superposition of the
-// monochromatic solutions, each with time dependence exp(-i omega_j t)
-// (Eq. fov4 advances a forward wave by exp(+i k dz)) -- by a radix-2
-// Stockham transform in shared memory.  A block handles `tx` consecutive x
-// of one band.
-template <typename C, typename R>
-__global__ void omega_to_t_kernel(const C* __restrict__ in, C* __restrict__ out, int nb,
-                                  int logb, int nx, int tx) {
-  extern __shared__ __align__(16) unsigned char sm[];
-  C* a = reinterpret_cast<C*>(sm);
-  C* b = a + size_t(tx) * nb;
-  const int band = blockIdx.y;
-  const int x0 = blockIdx.x * tx;
-  // load [nb][tx] -> a[xi][j]
-  for (int c = threadIdx.x; c < nb * tx; c += blockDim.x) {
-    const int j = c / tx, xi = c % tx;
-    a[xi * nb + j] = in[(size_t(j) * 2 + band) * nx + x0 + xi];
-  }
-  __syncthreads();
-  const int half = nb >> 1;
-  for (int ns = 1; ns < nb; ns <<= 1) {
-    for (int c = threadIdx.x; c < half * tx; c += blockDim.x) {
-      const int xi = c / half, j = c % half;
-      const int k = j % ns;
-      const C u = a[xi * nb + j];
-      C v = a[xi * nb + j + half];
-      // w = exp(-i pi k / ns)
-      R sw, cw;
-      if constexpr (sizeof(R) == 8) sincospi(double(k) / double(ns), &sw, &cw);
-      else sincospif(float(k) / float(ns), &sw, &cw);
-      v = C{v.x * cw + v.y * sw, v.y * cw - v.x * sw};
-      const int base = (j / ns) * ns * 2 + k;
-      b[xi * nb + base] = C{u.x + v.x, u.y + v.y};
-      b[xi * nb + base + ns] = C{u.x - v.x, u.y - v.y};
-    }
-    __syncthreads();
-    C* t = a;
-    a = b;
-    b = t;
-  }
-  for (int c = threadIdx.x; c < nb * tx; c += blockDim.x) {
-    const int xi = c / nb, m = c % nb;
-    out[(size_t(band) * nx + x0 + xi) * nb + m] = a[xi * nb + m];
-  }
-}
-
 // The coupling of Eq. fov10 alone, for a step of the coefficients (am1h,
 // bh) of each row: psi_+ <- psi_+ + (a-1) psi_+ + b e psi_-, psi_- <- psi_- +
 // (a-1) psi_- + b conj(e) psi_+ (old values on the right) inside the crystal
@@ -239,36 +192,6 @@ int launch_finish_f64(const double2* state, double2* out, const double* g, int n
                       cudaStream_t st) {
   return launch_finish(state, out, static_cast<float2*>(nullptr), g, n_rows, nx, dx, final_powers,
                        power_stride, scratch, st);
-}
-
-int launch_omega_to_t(const void* d_in, void* d_out, int nb, int nx, int precision,
-                      cudaStream_t st) {
-  int logb = 0;
-  while ((1 << logb) < nb) ++logb;
-  const size_t csize = precision == BPM_FP32_FUSED ? 8 : 16;
-  int tx = 1;
-  while (tx < 16 && size_t(tx) * 2 * nb * 2 * csize <= 96 * 1024 && (nx % (tx * 2)) == 0) tx *= 2;
-  const size_t smem = size_t(tx) * nb * 2 * csize;
-  dim3 grid(nx / tx, 2);
-  cudaError_t e;
-  if (precision == BPM_FP32_FUSED) {
-    auto k = omega_to_t_kernel<float2, float>;
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e == cudaSuccess) {
-      k<<<grid, 256, smem, st>>>(static_cast<const float2*>(d_in), static_cast<float2*>(d_out),
-                                 nb, logb, nx, tx);
-      e = cudaGetLastError();
-    }
-  } else {
-    auto k = omega_to_t_kernel<double2, double>;
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e == cudaSuccess) {
-      k<<<grid, 256, smem, st>>>(static_cast<const double2*>(d_in), static_cast<double2*>(d_out),
-                                 nb, logb, nx, tx);
-      e = cudaGetLastError();
-    }
-  }
-  return e == cudaSuccess ? BPM_OK : cuda_fail(e, "omega_to_t");
 }
 
 namespace {
