@@ -173,8 +173,11 @@ void phase_factors(const bpm_plan_s* plan, int steps, std::vector<double2>* out)
 // round-robin order (item i = row i mod B, chunk i div B).  Every launch is
 // full, each row's chunks run in order (item i + B lands in a later launch),
 // no row appears twice in a launch, and rows sweeping the same z-range share
-// their strain slices in L2.  A remainder shorter than a chunk runs as a
-// second round of the same kind.
+// their strain slices in L2.  A remainder shorter than a chunk is the rows' last
+// item in the same order where a CTA marches one row (nx >= 2048: it stops at
+// its row's last step); as a round of its own it left the GPU part empty twice
+// (256 rows x 4096 x 1000 steps 9.09 -> 8.88 ms).  With several rows per CTA,
+// whose steps are counted together, it is that second round.
 // Host-to-device upload on the march's stream: a plain async copy, or, while
 // the stream is being captured into a graph, kernel parameters (which the
 // graph keeps; a captured copy would re-read the host memory at replay).
@@ -204,22 +207,29 @@ static int launch_rotated(bpm_plan_s* plan, PlanAux* aux, const std::vector<RowD
   std::vector<RowDescF32> sched;
   struct Launch { size_t off; int count; int steps; };
   std::vector<Launch> launches;
-  auto round = [&](int c0, int c1, int len) {
+  auto round = [&](int c0, int c1) {
     const long items = long(nb) * (c1 - c0);
     for (long i = 0; i < items; i += resident) {
       const int cnt = int(std::min<long>(resident, items - i));
-      launches.push_back({sched.size(), cnt, len});
+      launches.push_back({sched.size(), cnt, 0});
       for (int k = 0; k < cnt; ++k) {
         const long it = i + k;
         RowDescF32 d = rows[it % nb];
-        d.n_begin = n_begin + int(c0 + it / nb) * chunk;
+        const int at = int(c0 + it / nb) * chunk, len = std::min(chunk, steps - at);
+        d.n_begin = n_begin + at;
         d.n_end = d.n_begin + len;
+        launches.back().steps = std::max(launches.back().steps, len);
         sched.push_back(d);
       }
     }
   };
-  round(0, full, chunk);
-  if (rem > 0) round(full, full + 1, rem);
+  const int pieces = full + (rem > 0);
+  if (plan->logn >= 11) {
+    round(0, pieces);
+  } else {
+    round(0, full);
+    if (rem > 0) round(full, pieces);
+  }
   const bool captured = capturing(st);
   if (aux->sched_cap < sched.size()) {
     if (captured)

@@ -232,6 +232,8 @@ __global__ void __launch_bounds__(F2Cfg<LOGN>::THREADS, F2Cfg<LOGN>::THREADS >= 
   const int row = blockIdx.x * C::ROWS + rl;
   const bool active = row < n_rows;
   const RowDescF32 d = rows[active ? row : 0];
+  // rows of a launch may have fewer steps left (the last chunk of a rotation)
+  if constexpr (C::ROWS == 1) steps = min(steps, d.n_end - d.n_begin);
   const bool lead = active && t == 0 && band == 0;
 
   float2* buf = reinterpret_cast<float2*>(smem + C::OFF_BUF) + (rl * 2 + band) * C::PADN;
