@@ -353,9 +353,10 @@ int bpm_march_f64_noalloc(void* d_psi, int32_t nx, int32_t n_rows, const void* d
  * step of Eq. fov10).  Rows of nx >= 64 march with 8 points per thread where
  * that is the faster form: one CTA per row up to nx = 512 (any number of rows
  * to nx = 128, 1000 rows of 256, 608 of 512) and for 137 to 304 rows of 1024,
- * spread over clusters of 8 or 16 CTAs else (nx = 1024 to 136 rows, 2048 to
- * 72, 4096 to 36, 8192 to 28, 16384 always but for 15 rows); they report the
- * code below that their size and splitting had as single rows.  *layout = 10
+ * spread over clusters of 8 or 16 CTAs else (nx = 1024 to 136 rows; 2048 from
+ * 72 rows, 4096 from 36, 8192 from 15, 16384 from 7 on in rotation, up to about
+ * 1.5 times these rows, or more where the other forms need further waves);
+ * they report the code below that their size and splitting had as single rows.  *layout = 10
  * the Forest-Ruth step on one cluster per row (512 <= nx <= 4096), 9 the
  * Forest-Ruth step on one cluster per row (nx = 4096 and 8192: 4-CTA
  * half-band split, split band), 8 the nx = 4096 half-band split with 16

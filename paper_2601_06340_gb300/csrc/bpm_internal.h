@@ -391,6 +391,8 @@ int launch_spread(int logn, int lc, int split, const RowDescF32* d_rows, int n_r
                   const float4* d_tw, int* d_status, cudaStream_t st);
 int spread_capacity(int logn, int lc, int split);   // clusters resident at once
 int spread_choice(int logn, int rows, int split);   // lc of a launch, 0: not spread
+// how many steps of a full launch of spread rows the other form's step takes
+double spread_limit(int logn, int rows, int split);
 int fused_threads(int logn);
 
 }  // namespace bpm

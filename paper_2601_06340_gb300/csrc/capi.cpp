@@ -88,6 +88,15 @@ bool spread_rows(const bpm_plan_s* plan) {
   return false;
 }
 
+// Whether with some splitting they are more than a launch keeps resident.
+bool spread_rotates(const bpm_plan_s* plan) {
+  for (int s : {BPM_SPLIT_FIRST_ORDER, BPM_SPLIT_VERLET, BPM_SPLIT_FOREST_RUTH}) {
+    const int lc = spread_choice(plan->logn, plan->nb, s);
+    if (lc > kOneCta && plan->nb > spread_capacity(plan->logn, lc, s)) return true;
+  }
+  return false;
+}
+
 }  // namespace
 
 inline PlanAux* aux_of(bpm_plan_s* plan) { return &plan->aux; }
@@ -199,7 +208,7 @@ static int upload(void* dst, const void* src, size_t bytes, cudaStream_t st, boo
 
 static int launch_rotated(bpm_plan_s* plan, PlanAux* aux, const std::vector<RowDescF32>& rows,
                           int n_begin, int steps, int resident, cudaStream_t st, int chunk = 0,
-                          int layout = -1) {
+                          int layout = -1, int spread = 0) {
   const int nb = plan->nb;
   if (chunk <= 0) chunk = std::max(std::min(steps, 64), steps / 24);
   chunk = std::min(chunk, steps);
@@ -247,9 +256,12 @@ static int launch_rotated(bpm_plan_s* plan, PlanAux* aux, const std::vector<RowD
                    "upload launch schedule");
   if (urc != BPM_OK) return urc;
   for (const Launch& l : launches) {
-    int rc = launch_fused_layout(plan->logn, aux->d_sched + l.off, l.count, l.steps,
-                                 static_cast<const float4*>(plan->d_tw), plan->d_status, st,
-                                 layout);
+    const RowDescF32* d_rows = aux->d_sched + l.off;
+    const float4* tw = static_cast<const float4*>(plan->d_tw);
+    int rc = spread ? launch_spread(plan->logn, spread, plan->split, d_rows, l.count, l.steps, tw,
+                                    plan->d_status, st)
+                    : launch_fused_layout(plan->logn, d_rows, l.count, l.steps, tw,
+                                          plan->d_status, st, layout);
     if (rc != BPM_OK) return rc;
   }
   return BPM_OK;
@@ -333,11 +345,40 @@ static bool fr_staged(const bpm_plan_s* plan) {
   return fv && std::strcmp(fv, "staged") == 0;
 }
 
+// The chunk in which more spread rows than fit at once rotate (the march's
+// steps if no chunk beats plain waves): the fewest steps over all launches,
+// a launch's start counted as kSpreadStart steps.  At most kSpreadPieces
+// chunks a row, which bounds the launch schedule.
+constexpr int kSpreadPieces = 24, kSpreadStart = 4;
+
+static int spread_chunk(int rows, int cap, int steps, double* cost) {
+  int best = steps;
+  *cost = 1e30;
+  for (int k = 1; k <= kSpreadPieces; ++k) {
+    const int chunk = (steps + k - 1) / k, pieces = (steps + chunk - 1) / chunk;
+    if (k > 1 && chunk < 32) break;
+    const double c = double((long(rows) * pieces + cap - 1) / cap) * (chunk + kSpreadStart);
+    if (c < *cost) {
+      *cost = c;
+      best = chunk;
+    }
+  }
+  return best;
+}
+
 // log2 of the CTAs that each row of a plan is spread over, 0 if not (any
-// BPM_FUSED_LAYOUT forces the other forms).
-static int spread_lc(const bpm_plan_s* plan) {
+// BPM_FUSED_LAYOUT forces the other forms), and the chunk if they rotate.
+static int spread_lc(const bpm_plan_s* plan, int steps, int* chunk = nullptr) {
   if (!plan->d_prop_nat || std::getenv("BPM_FUSED_LAYOUT")) return 0;
-  return spread_choice(plan->logn, plan->nb, plan->split);
+  const int lc = spread_choice(plan->logn, plan->nb, plan->split);
+  const int cap = lc > kOneCta ? spread_capacity(plan->logn, lc, plan->split) : 0;
+  if (cap > 0 && plan->nb > cap) {
+    double cost = 0.0;
+    const int c = spread_chunk(plan->nb, cap, steps, &cost);
+    if (cost > spread_limit(plan->logn, plan->nb, plan->split) * steps + kSpreadStart) return 0;
+    if (chunk) *chunk = c;
+  }
+  return lc;
 }
 
 static LaunchShape choose_layout(bpm_plan_s* plan, PlanAux* aux, const void* state, int n_begin,
@@ -345,11 +386,14 @@ static LaunchShape choose_layout(bpm_plan_s* plan, PlanAux* aux, const void* sta
 
 static LaunchShape choose_shape(bpm_plan_s* plan, PlanAux* aux, const void* state, int n_begin,
                                 int steps, cudaStream_t st) {
-  const int lc = spread_lc(plan);
+  int chunk = 0;
+  const int lc = spread_lc(plan, steps, &chunk);
   if (lc == 0) return choose_layout(plan, aux, state, n_begin, steps, st);
   // reported under the codes of the cluster layouts (bpm_launch_shape)
   LaunchShape sh;
   sh.spread = lc;
+  sh.chunk = chunk;
+  sh.rotated = chunk > 0 && chunk < steps;
   const int logn = plan->logn;
   if (plan->split == BPM_SPLIT_VERLET)
     sh.layout = logn >= 12               ? kLayoutSplit4Half
@@ -658,7 +702,7 @@ static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, const MarchInput& in, v
                      n_begin, n_end, st);
     return rc == BPM_OK ? finish() : rc;
   }
-  if (fr_staged(plan) && spread_lc(plan) == 0) {
+  if (fr_staged(plan) && spread_lc(plan, steps) == 0) {
     rc = stage_march(plan, aux, in, state, g, nullptr, 0, st, captured);
     if (rc == BPM_OK)
       rc = march_staged_fr(plan, aux, state, d_rec, d_pw, n_begin, n_end, captured, st);
@@ -671,7 +715,7 @@ static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, const MarchInput& in, v
   // the search for a batch's launch shape marches trials from the state
   // buffer, so the input goes there first
   MarchInput from = in;
-  if (spread_lc(plan) == 0 && plan->nb > 1) {
+  if (spread_lc(plan, steps) == 0 && plan->nb > 1) {
     rc = copy_input(in, state, st);
     if (rc != BPM_OK) return rc;
     from.src = state;
@@ -694,10 +738,11 @@ static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, const MarchInput& in, v
                    : launch_fused_layout(plan->logn, d_rows, plan->nb, steps, tw, plan->d_status,
                                          st, sh.layout);
   } else {
-    const int cap = sh.layout == kLayoutCtaHalf ? fused_half_capacity(plan->logn)
+    const int cap = sh.spread                     ? spread_capacity(plan->logn, sh.spread, plan->split)
+                    : sh.layout == kLayoutCtaHalf ? fused_half_capacity(plan->logn)
                     : sh.layout == kLayoutCtaFR ? fused_fr_capacity(plan->logn)
                                                 : fused_launch_capacity(plan->logn, false);
-    rc = launch_rotated(plan, aux, rows, n_begin, steps, cap, st, sh.chunk, sh.layout);
+    rc = launch_rotated(plan, aux, rows, n_begin, steps, cap, st, sh.chunk, sh.layout, sh.spread);
   }
   return rc == BPM_OK ? finish() : rc;
 }
@@ -750,6 +795,7 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
   compute_energy_consts(plan.get());
 
   bpm_plan_s* pl = plan.get();
+  PlanAux* aux = aux_of(pl);
   const size_t n = plane_of(pl), nb = pl->nb, cs = csize(pl);
   const bool vol = pl->ny > 1;
   int rc = BPM_OK;
@@ -764,6 +810,12 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
   if (half_split)
     A(&pl->d_prop_split, nb * size_t(split_table_stride(pl, 11)) * cs, "split propagator tables");
   if (spread_rows(pl)) A(&pl->d_prop_nat, nb * 2 * n * cs, "natural propagator tables");
+  // (a capture must find the schedule of rotating spread rows in place)
+  if (pl->d_prop_nat && spread_rotates(pl)) {
+    aux->sched_cap = nb * kSpreadPieces;
+    A(reinterpret_cast<void**>(&aux->d_sched), aux->sched_cap * sizeof(RowDescF32),
+      "launch schedule");
+  }
   const bool f64 = f64_fused(pl);
   A(&pl->d_tw, (f64 ? f64_twiddle_count(pl) : size_t(pl->nx)) * 16, "twiddles");
   if (vol) {
@@ -780,7 +832,6 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
   A(&pl->d_finish, fin_bytes, "finish scratch");
   A(&pl->d_io, nb * 2 * n * 16, "host staging");
   A(reinterpret_cast<void**>(&pl->d_status), sizeof(int), "status");
-  PlanAux* aux = aux_of(pl);
   A(reinterpret_cast<void**>(&aux->d_g), nb * sizeof(double2), "phase factors");
   if (rc == BPM_OK) {
     e = cudaStreamCreateWithFlags(&aux->stream, cudaStreamNonBlocking);

@@ -299,6 +299,8 @@ __global__ void __launch_bounds__((SpreadCfg<LOGN, LC>::T), 1)
   const int c = int(cluster.block_rank());
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const RowDescF32 d = rows[blockIdx.x / C];
+  // rows of a launch may have fewer steps left (the last chunk of a rotation)
+  steps = min(steps, d.n_end - d.n_begin);
   const bool lead = t == 0;
 
   // thread number -> hi, u = (band, column), position in the column and row

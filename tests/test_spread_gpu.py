@@ -30,12 +30,12 @@ METHOD = {FIRST: "first_order", VERLET: "verlet", FR: "forest_ruth"}
 NZ, EVERY = 40, 7
 
 
-def _workload(nx, rows):
+def _workload(nx, rows, nz=NZ):
     rng = np.random.default_rng(nx + rows)
-    wl = inputs.pulse_batched(nx=nx, nz=NZ, n_energy=rows, dx_um=0.4, record_every=EVERY)
+    wl = inputs.pulse_batched(nx=nx, nz=nz, n_energy=rows, dx_um=0.4, record_every=EVERY)
     wl.psi0 = rng.standard_normal((rows, 2, nx)) + 1j * rng.standard_normal((rows, 2, nx))
-    wl.crystal = dict(kind=inputs.CRYSTAL_MASK, mask=(rng.uniform(size=(NZ, nx)) < 0.8))
-    wl.strain = dict(kind=inputs.STRAIN_ARRAY, ux=rng.uniform(-1e-3, 1e-3, (NZ, nx)))
+    wl.crystal = dict(kind=inputs.CRYSTAL_MASK, mask=(rng.uniform(size=(nz, nx)) < 0.8))
+    wl.strain = dict(kind=inputs.STRAIN_ARRAY, ux=rng.uniform(-1e-3, 1e-3, (nz, nx)))
     return wl
 
 
@@ -55,6 +55,24 @@ def test_spread_matches_oracle(bpm_lib, monkeypatch, nx, rows, split):
     pick = sorted({0, rows // 2, rows - 1})
     ref = run_ref(wl, method=METHOD[split], rows=pick)
     tol = 7.2e-6 if split == FR else 2.4e-6
+    errs = band_errors(out.psi[pick], ref.psi, out.records[pick], ref.records)
+    assert max(errs) <= tol, errs
+    assert np.allclose(out.powers[pick], ref.powers, rtol=1e-5)
+
+
+@pytest.mark.parametrize("split", [FIRST, VERLET, FR])
+@pytest.mark.parametrize("nx,rows", [(2048, 90), (4096, 45), (8192, 17), (16384, 8)])
+def test_rotating_rows_match_oracle(bpm_lib, monkeypatch, nx, rows, split):
+    """More rows than a launch keeps resident, in chunks with a shorter last
+    one: 151 steps, so twice the bound of 40 (random walk)."""
+    monkeypatch.delenv("BPM_FUSED_LAYOUT", raising=False)
+    wl = _workload(nx, rows, 151)
+    with binding.Plan(wl, binding.BPM_FP32_FUSED, splitting=split) as plan:
+        out = plan.propagate()
+        assert 0 < binding.bpm_launch_shape(plan.handle)[1] < 151
+    pick = [0, rows - 1]
+    ref = run_ref(wl, method=METHOD[split], rows=pick)
+    tol = 14.4e-6 if split == FR else 4.8e-6
     errs = band_errors(out.psi[pick], ref.psi, out.records[pick], ref.records)
     assert max(errs) <= tol, errs
     assert np.allclose(out.powers[pick], ref.powers, rtol=1e-5)
