@@ -44,8 +44,7 @@ WORKLOAD = ("bragg_bent: 2D symmetric Bragg, bent crystal R=1 m nu=0.28, 8 keV, 
 FLOPS_PER_CELL = lambda n: 4 * 5 * math.log2(n)      # 4 FFTs x 5 N log2 N / N
 # the single-solve march kernel by launch layout (bpm_launch_shape): name, SMs
 MARCH_KERNELS = {
-    2: ("fused4s_march_kernel (4-CTA cluster per solve: two half-band parts per band, "
-        "8 points per thread)", 4),
+    2: ("spread_march_kernel<12, 4> (16-CTA cluster per solve, 8 points per thread)", 16),
     8: ("fused4e_march_kernel<11> (4-CTA cluster per solve: two half-band parts per band, "
         "16 points per thread)", 4),
     1: ("fused3_march_kernel<12> (2-CTA cluster per solve, one band per CTA)", 2),
@@ -53,11 +52,8 @@ MARCH_KERNELS = {
 }
 
 KERNEL_SOURCES = ["paper_2601_06340_gb300/csrc/radix.cuh",
-                  "paper_2601_06340_gb300/csrc/fused4s_kernel.cuh",
                   "paper_2601_06340_gb300/csrc/fused_kernel.cuh",
-                  "paper_2601_06340_gb300/csrc/fused2_kernel.cuh",
-                  "paper_2601_06340_gb300/csrc/fused3_kernel.cuh",
-                  "paper_2601_06340_gb300/csrc/fused4_kernel.cuh"]
+                  "paper_2601_06340_gb300/csrc/spread_kernel.cuh"]
 
 
 def kernel_hash() -> str:
@@ -412,7 +408,7 @@ def volume_run(dev, stream, barrier, max_over_ranks, world, rank, ref=None, step
     out = {"workload": "cube_dislocation_3d: Si(440)-like at 17.45 keV, 10 um box crystal, "
                        "edge dislocation along y, Nx=512, Ny=256, Nz=300, dx=dy=dz=0.05 um",
            "value": world * wv.cell_updates / (ms * 1e-3), "unit": UNIT, "ms_per_march": ms,
-           "launches_per_march": 2 * wv.nz + 2, "l2": L2_NOTE,
+           "launches_per_march": 3, "l2": L2_NOTE,
            "paper_context": {"seconds": 13.0, "grid": "300 x 200 x 300",
                              "hardware": "one Perlmutter node (CPU vs GPU not stated)"}}
     if ref is not None:
@@ -440,7 +436,7 @@ def configs_run(dev, stream, barrier, max_over_ranks, world, rank, refs=None, st
         row = {"nx": wl.nx, "nz": wl.nz}
         psi = {}
         for prec, key in ((binding.BPM_FP32_FUSED, "fused_fp32"),
-                          (binding.BPM_FP64_PLAIN, "plain_fp64")):
+                          (binding.BPM_FP64_PLAIN, "fp64")):
             plan = binding.Plan(wl, prec)
             dt = torch.complex64 if prec == binding.BPM_FP32_FUSED else torch.complex128
             x = torch.from_numpy(wl.psi0).to(dev).to(dt)
@@ -459,12 +455,12 @@ def configs_run(dev, stream, barrier, max_over_ranks, world, rank, refs=None, st
                         "ms_per_march": ms}
             psi[key] = y.cpu().numpy().astype(np.complex128)
             plan.close()
-        row["fused_speedup"] = row["fused_fp32"]["value"] / row["plain_fp64"]["value"]
+        row["fused_speedup"] = row["fused_fp32"]["value"] / row["fp64"]["value"]
         if refs:
             ref, cpu_s = refs[name].result()
             row["oracle_1core"] = {"value": wl.cell_updates / cpu_s, "unit": UNIT, "cores": 1}
             row["fused_fp32"]["rel_l2_err"] = rel_l2_bands(psi["fused_fp32"], ref.psi)
-            row["plain_fp64"]["rel_l2_err"] = rel_l2_bands(psi["plain_fp64"], ref.psi)
+            row["fp64"]["rel_l2_err"] = rel_l2_bands(psi["fp64"], ref.psi)
         out[name] = row
     out["l2"] = L2_NOTE
     return out
@@ -728,26 +724,50 @@ def run_gpu(args, rks):
     # the oracle's references, computed on the host from here on
     submit_jobs()
 
-    # ---- plain FP64 per-step GPU path (same workload) ----------------------
+    # ---- FP64 plan: one cooperative launch per march (same workload) --------
     plan64 = binding.Plan(wl, FP64)
     x64 = torch.from_numpy(wl.psi0).to(dev)
     y64 = torch.empty_like(x64)
-    binding.bpm_propagate_device(plan64.handle, x64, y64, None, None, 0, wl.nz,
-                                 stream.cuda_stream)
-    barrier()
     s64 = max(1, args.steps // 5)
-    ev64 = timed_ms(lambda: binding.bpm_propagate_device(plan64.handle, x64, y64, None, None,
-                                                         0, wl.nz, stream.cuda_stream),
-                    s64, stream, flush)
+
+    def march64():
+        binding.bpm_propagate_device(plan64.handle, x64, y64, None, None, 0, wl.nz,
+                                     stream.cuda_stream)
+    march64()
+    barrier()
+    ev64 = timed_ms(march64, s64, stream, flush)
     barrier()
     ms64 = max_over_ranks(sum(elapsed(ev64))) / s64
     value64 = world * cells / (ms64 * 1e-3)
     psi64 = y64.cpu().numpy()
+
+    # ---- plain FP64 per-step GPU path (same workload): a kernel per pass, on
+    # the caller's tables, no common phase -------------------------------------
+    from oracle import run as orun
+    con = orun.plans_for(wl)[0]
+    d_prop = torch.from_numpy(np.stack([con.prop_plus, con.prop_minus])[None] / wl.nx).to(dev)
+    d_ab = torch.from_numpy(np.array([[con.a, con.b]], dtype=np.complex128)).to(dev)
+    d_ph = torch.from_numpy(np.ascontiguousarray(plan64.slices()[1])).to(dev)
     plan64.close()
+
+    def plain64():
+        y64.copy_(x64)
+        binding.bpm_march_f64_noalloc(y64, wl.nx, 1, d_prop, d_ab, d_ph, 0, wl.nz,
+                                      stream.cuda_stream)
+    plain64()
+    barrier()
+    evp64 = timed_ms(plain64, s64, stream, flush)
+    barrier()
+    msp64 = max_over_ranks(sum(elapsed(evp64))) / s64
+    valuep64 = world * cells / (msp64 * 1e-3)
+    ang = math.fmod(wl.nz * math.fmod(con.dzh * con.c, 2 * math.pi), 2 * math.pi)
+    psip64 = y64.cpu().numpy() * complex(math.cos(ang), math.sin(ang))
+    del d_prop, d_ab, d_ph
     # ---- parity on the timed workload (the oracle's reference) -------------
     ref = jobs["head"].result()[0] if "head" in jobs else None
     err32 = rel_l2_bands(fused_psi, ref.psi) if ref is not None else None
     err64 = rel_l2_bands(psi64, ref.psi) if ref is not None else None
+    errp64 = rel_l2_bands(psip64, ref.psi) if ref is not None else None
 
     # ---- batched: 256 photon energies (pulse), one launch + energy->time --
     batched = None
@@ -842,7 +862,7 @@ def run_gpu(args, rks):
     achieved = cells * FLOPS_PER_CELL(wl.nx) / avg_launch_s / 1e12
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
                 "frac": achieved / peak_tflops,
-                "traffic": profiled_traffic("fused_march_bragg_bent.md"),
+                "traffic": profiled_traffic("spread_march_bragg_bent.md"),
                 "kernel": MARCH_KERNELS[march_layout][0],
                 "peak_basis": "measured: FP32 FMA throughput kernel (bpm_fp_peak, the faster "
                               "of FFMA and packed FFMA2) on this GPU in this run",
@@ -885,17 +905,25 @@ def run_gpu(args, rks):
             "tolerance": 2e-4,
             "latency_ms": {"p50": float(np.percentile(lat, 50)),
                            "p99": float(np.percentile(lat, 99))},
-            "fp64_plain": {"value": value64, "unit": UNIT, "ms_per_step": ms64,
-                           "rel_l2_err": err64, "tolerance": 1e-10,
-                           "fused_speedup": value / value64,
+            "fp64_plain": {"value": valuep64, "unit": UNIT, "ms_per_step": msp64,
+                           "rel_l2_err": errp64, "tolerance": 1e-10,
+                           "fused_speedup": value / valuep64,
                            "roofline": {"bound": "fp64 alu / launches",
-                                        "achieved": value64 * FLOPS_PER_CELL(wl.nx) / 1e12,
+                                        "achieved": valuep64 * FLOPS_PER_CELL(wl.nx) / 1e12,
                                         "peak": peaks["fp64_tflops"], "unit": "TFLOP/s",
-                                        "frac": value64 * FLOPS_PER_CELL(wl.nx) / 1e12
+                                        "frac": valuep64 * FLOPS_PER_CELL(wl.nx) / 1e12
                                         / peaks["fp64_tflops"],
                                         "launches_per_step": 2 * (wl.nx.bit_length() // 2) + 2,
                                         "peak_basis": "measured: FP64 DFMA throughput kernel "
                                                       "(bpm_fp_peak)"}},
+            "fp64_plan": {"value": value64, "unit": UNIT, "ms_per_step": ms64,
+                          "rel_l2_err": err64, "tolerance": 1e-10,
+                          "how": "f64_march_kernel: the march in one cooperative launch",
+                          "roofline": {"bound": "fp64 latency / grid barriers",
+                                       "achieved": value64 * FLOPS_PER_CELL(wl.nx) / 1e12,
+                                       "peak": peaks["fp64_tflops"], "unit": "TFLOP/s",
+                                       "frac": value64 * FLOPS_PER_CELL(wl.nx) / 1e12
+                                       / peaks["fp64_tflops"]}},
             "peaks": peaks,
             "batched": batched,
             "configs": configs,
@@ -905,7 +933,7 @@ def run_gpu(args, rks):
             "serving": serving,
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h},
-            "gpu_launches": 2 * args.steps,
+            "gpu_launches": 3 * args.steps,   # start, march, finish
             "roofline": roofline,
             "cpu_baseline": cpu_baseline,
             "clocks": clocks,

@@ -40,6 +40,29 @@ int spread_capacity(int logn, int lc, int split) {
   return 0;
 }
 
+// The other form's step over that of a full spread launch, first order (the
+// splitting forms): N = 2048 2.89 over 1.88 us (3.58 over 2.11; 9.6 over 5.8) up
+// to a row per SM, 4.8 over 1.88 beyond; N = 4096 3.56 over 1.97 (5.28 over 2.33;
+// 12.3 over 6.5) up to the 2-CTA cluster's 76 rows, 5.1 over 1.97 beyond; N =
+// 8192 5.03 over 2.10 (6.9 over 2.52; 18.7 over 6.7) and N = 16384 7.4 over 2.96
+// (9.1 over 3.34) per wave of the split band's 36 and 15 clusters, Forest-Ruth
+// N = 16384 117 over 9.1.  The limits lie below by the launches' starts: in rotation
+// 101 rows of 2048 2.65 against 2.90, 57 of 4096 3.31 against 3.57.
+double spread_limit(int logn, int rows, int split) {
+  const bool first = split == BPM_SPLIT_FIRST_ORDER;
+  auto waves = [&] {
+    const int cap = std::max(1, fused_launch_capacity(logn, true));
+    return (rows + cap - 1) / cap;
+  };
+  switch (logn) {
+    case 11: return 2 * rows > fused_launch_capacity(11, false) ? 2.45 : first ? 1.5 : 1.6;
+    case 12: return waves() > 1 ? 2.4 : first ? 1.7 : 1.8;
+    case 13: return waves() * (first ? 2.3 : 2.6);
+    case 14: return split == BPM_SPLIT_FOREST_RUTH ? 12.0 * waves() : 2.4 * waves();
+    default: return 1.0;
+  }
+}
+
 // Which rows take 8 points per thread, and over how many CTAs (log2, or
 // kOneCta; 0: the kernels of 16 points that keep a row on one to eight SMs).
 // More rows than spread_capacity clusters march in rotation (rotated launches
@@ -64,29 +87,6 @@ int spread_capacity(int logn, int lc, int split) {
 //              band 7.1 alone, 7.7 at 15 rows, 14.4 at 16).
 // The splitting forms gain more at every size (Verlet N = 2048 3.55 -> 1.51,
 // Forest-Ruth N = 16384 stage by stage 114 -> 9.5).
-// The other form's step over that of a full spread launch, first order (the
-// splitting forms): N = 2048 2.89 over 1.88 us (3.58 over 2.11; 9.6 over 5.8) up
-// to a row per SM, 4.8 over 1.88 beyond; N = 4096 3.56 over 1.97 (5.28 over 2.33;
-// 12.3 over 6.5) up to the 2-CTA cluster's 76 rows, 5.1 over 1.97 beyond; N =
-// 8192 5.03 over 2.10 (6.9 over 2.52; 18.7 over 6.7) and N = 16384 7.4 over 2.96
-// (9.1 over 3.34) per wave of the split band's 36 and 15 clusters, Forest-Ruth
-// N = 16384 117 over 9.1.  The limits lie below by the launches' starts: in rotation
-// 101 rows of 2048 2.65 against 2.90, 57 of 4096 3.31 against 3.57.
-double spread_limit(int logn, int rows, int split) {
-  const bool first = split == BPM_SPLIT_FIRST_ORDER;
-  auto waves = [&] {
-    const int cap = std::max(1, fused_launch_capacity(logn, true));
-    return (rows + cap - 1) / cap;
-  };
-  switch (logn) {
-    case 11: return 2 * rows > fused_launch_capacity(11, false) ? 2.45 : first ? 1.5 : 1.6;
-    case 12: return waves() > 1 ? 2.4 : first ? 1.7 : 1.8;
-    case 13: return waves() * (first ? 2.3 : 2.6);
-    case 14: return split == BPM_SPLIT_FOREST_RUTH ? 12.0 * waves() : 2.4 * waves();
-    default: return 1.0;
-  }
-}
-
 int spread_choice(int logn, int rows, int split) {
   auto cap = [&](int lc) { return spread_capacity(logn, lc, split); };
   switch (logn) {
