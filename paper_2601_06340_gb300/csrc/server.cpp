@@ -74,6 +74,8 @@ struct Request {
   void* d_rec = nullptr;
   double* d_pow = nullptr;
   double2* d_g = nullptr;
+  void* d_fin = nullptr;       // launch_finish scratch (the plan's may be in use by a march
+                               // of the plan on a caller's stream)
   double2* d_out = nullptr;    // c128 staging
   cudaEvent_t ready = nullptr; // staged and prepared on io_stream
   cudaEvent_t out_ev = nullptr;   // results copied to the pinned staging
@@ -152,7 +154,8 @@ size_t footprint_of(const bpm_plan_s* p, bool need_rec) {
   size_t b = nb * 2 * n * cs                       // state
              + nb * 2 * n * 16                     // c128 output staging
              + nb * size_t(p->n_rec + 1) * 2 * 8   // powers
-             + nb * 16;                            // phase factors
+             + nb * 16                             // phase factors
+             + finish_scratch_bytes(p->nb, p->nx);
   if (need_rec) b += nb * size_t(p->n_rec) * 2 * n * cs;
   if (!slices_resident(p)) b += slice_data_bytes(p);
   return b;
@@ -195,12 +198,13 @@ void release(Server& s, Request& r) {
     cudaEventDestroy(r.ready);
     r.ready = nullptr;
   }
-  void* ptrs[] = {r.d_state, r.d_rec, r.d_pow, r.d_g, r.d_out};
+  void* ptrs[] = {r.d_state, r.d_rec, r.d_pow, r.d_g, r.d_fin, r.d_out};
   for (void* p : ptrs)
     if (p) cudaFreeAsync(p, s.io_stream);
   r.d_state = r.d_rec = nullptr;
   r.d_pow = nullptr;
   r.d_g = r.d_out = nullptr;
+  r.d_fin = nullptr;
 }
 
 // Allocate and stage a request (stream-ordered on io_stream).
@@ -230,7 +234,10 @@ int admit_device(Server& s, Request& r) {
   if (r.records && p->n_rec > 0) A(&r.d_rec, nb * size_t(p->n_rec) * 2 * n * cs);
   A(reinterpret_cast<void**>(&r.d_pow), nb * size_t(p->n_rec + 1) * 2 * 8);
   A(reinterpret_cast<void**>(&r.d_g), nb * 16);
+  const size_t fin_bytes = finish_scratch_bytes(p->nb, p->nx);
+  A(&r.d_fin, fin_bytes);
   A(reinterpret_cast<void**>(&r.d_out), nb * 2 * n * 16);
+  if (e == cudaSuccess) e = cudaMemsetAsync(r.d_fin, 0, fin_bytes, st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return e == cudaErrorMemoryAllocation ? BPM_ERR_OOM : BPM_ERR_CUDA;
@@ -274,11 +281,11 @@ int retire_enqueue(Server& s, Request& r) {
   if (p->precision == BPM_FP32_FUSED)
     rc = launch_finish_f32(static_cast<const float2*>(r.d_state), r.d_out, nullptr,
                            reinterpret_cast<const double*>(r.d_g), p->nb, p->nx, p->dx_um,
-                           r.d_pow + 2 * p->n_rec, pw_stride, p->d_finish, st);
+                           r.d_pow + 2 * p->n_rec, pw_stride, r.d_fin, st);
   else
     rc = launch_finish_f64(static_cast<const double2*>(p->d_state), r.d_out,
                            reinterpret_cast<const double*>(r.d_g), p->nb, p->nx, p->dx_um,
-                           r.d_pow + 2 * p->n_rec, pw_stride, p->d_finish, st);
+                           r.d_pow + 2 * p->n_rec, pw_stride, r.d_fin, st);
   if (rc != BPM_OK) return rc;
   char* h = static_cast<char*>(r.h_stage);
   e = cudaMemcpyAsync(h, r.d_out, nb * 2 * n * 16, cudaMemcpyDeviceToHost, st);
