@@ -60,6 +60,15 @@ void free_plan_memory(bpm_plan_s* plan) {
   }
   if (plan->d_status) cudaFree(plan->d_status);
   plan->d_status = nullptr;
+  PlanAux& aux = plan->aux;
+  for (void* p : {aux.d_rec, static_cast<void*>(aux.d_pow), static_cast<void*>(aux.d_g),
+                  static_cast<void*>(aux.d_sched)})
+    if (p) cudaFree(p);
+  aux.d_rec = nullptr;
+  aux.d_pow = nullptr;
+  aux.d_g = nullptr;
+  aux.d_sched = nullptr;
+  aux.rec_bytes = aux.pow_bytes = aux.sched_cap = 0;
 }
 
 size_t csize(const bpm_plan_s* plan) { return plan->precision == BPM_FP32_FUSED ? 8 : 16; }
@@ -942,7 +951,6 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
   }
   if (rc != BPM_OK) {
     if (aux->stream) cudaStreamDestroy(aux->stream);
-    if (aux->d_g) cudaFree(aux->d_g);
     free_plan_memory(pl);
     return rc;
   }
@@ -1468,10 +1476,6 @@ int bpm_destroy(bpm_plan_t plan) {
     cudaStreamSynchronize(aux->stream);
     cudaStreamDestroy(aux->stream);
   }
-  if (aux->d_rec) cudaFree(aux->d_rec);
-  if (aux->d_pow) cudaFree(aux->d_pow);
-  if (aux->d_g) cudaFree(aux->d_g);
-  if (aux->d_sched) cudaFree(aux->d_sched);
   free_plan_memory(plan);
   delete plan;
   return BPM_OK;
