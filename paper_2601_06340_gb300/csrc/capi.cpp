@@ -390,14 +390,25 @@ static int spread_lc(const bpm_plan_s* plan, int steps, int* chunk = nullptr) {
   return lc;
 }
 
-static LaunchShape choose_layout(bpm_plan_s* plan, PlanAux* aux, const void* state, int n_begin,
+// The input field to a state buffer by itself (a copy, or the conversion).
+static int copy_input(const MarchInput& in, void* state, cudaStream_t st) {
+  if (in.src == state) return BPM_OK;
+  if (in.kind == MarchInput::kC128ToC64)
+    return launch_convert_in(static_cast<const double2*>(in.src), static_cast<float2*>(state), in.n,
+                             st);
+  const size_t bytes = in.n * (in.kind == MarchInput::kC64 ? 8 : 16);
+  cudaError_t e = cudaMemcpyAsync(state, in.src, bytes, cudaMemcpyDeviceToDevice, st);
+  return e == cudaSuccess ? BPM_OK : cuda_fail(e, "copy input");
+}
+
+static LaunchShape choose_layout(bpm_plan_s* plan, PlanAux* aux, const MarchInput& in, int n_begin,
                                  int steps, cudaStream_t st);
 
-static LaunchShape choose_shape(bpm_plan_s* plan, PlanAux* aux, const void* state, int n_begin,
+static LaunchShape choose_shape(bpm_plan_s* plan, PlanAux* aux, const MarchInput& in, int n_begin,
                                 int steps, cudaStream_t st) {
   int chunk = 0;
   const int lc = spread_lc(plan, steps, &chunk);
-  if (lc == 0) return choose_layout(plan, aux, state, n_begin, steps, st);
+  if (lc == 0) return choose_layout(plan, aux, in, n_begin, steps, st);
   // reported under the codes of the cluster layouts (bpm_launch_shape)
   LaunchShape sh;
   sh.spread = lc;
@@ -418,7 +429,7 @@ static LaunchShape choose_shape(bpm_plan_s* plan, PlanAux* aux, const void* stat
   return sh;
 }
 
-static LaunchShape choose_layout(bpm_plan_s* plan, PlanAux* aux, const void* state, int n_begin,
+static LaunchShape choose_layout(bpm_plan_s* plan, PlanAux* aux, const MarchInput& in, int n_begin,
                                  int steps, cudaStream_t st) {
   NvtxRange nvtx("bpm_launch_shape_search");
   LaunchShape rule;
@@ -551,7 +562,12 @@ static LaunchShape choose_layout(bpm_plan_s* plan, PlanAux* aux, const void* sta
     cudaGetLastError();
     return rule;
   }
-  cudaMemcpyAsync(scratch, state, bytes, cudaMemcpyDeviceToDevice, st);
+  // (the trials march a copy: the input is staged with the row descriptors of
+  // the shape that they choose)
+  if (copy_input(in, scratch, st) != BPM_OK) {
+    cudaFreeAsync(scratch, st);
+    return rule;
+  }
   // another shape replaces the rule's only if it is at least 2% faster
   // (run-to-run noise of the trials is below 1%)
   LaunchShape best = cands.front();
@@ -636,17 +652,6 @@ static int march_staged_fr(bpm_plan_s* plan, PlanAux* aux, void* state, void* d_
   return rc;
 }
 
-// The input field to the state buffer by itself (a copy, or the conversion).
-static int copy_input(const MarchInput& in, void* state, cudaStream_t st) {
-  if (in.src == state) return BPM_OK;
-  if (in.kind == MarchInput::kC128ToC64)
-    return launch_convert_in(static_cast<const double2*>(in.src), static_cast<float2*>(state), in.n,
-                             st);
-  const size_t bytes = in.n * (in.kind == MarchInput::kC64 ? 8 : 16);
-  cudaError_t e = cudaMemcpyAsync(state, in.src, bytes, cudaMemcpyDeviceToDevice, st);
-  return e == cudaSuccess ? BPM_OK : cuda_fail(e, "copy input");
-}
-
 // The start of a march: the input to the state buffer, the phase factors and
 // the row descriptors (may be empty) to the device -- in one launch for few
 // rows, else a copy and two uploads.
@@ -721,23 +726,13 @@ static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, const MarchInput& in, v
   fused_rows(plan, static_cast<float2*>(state), static_cast<float2*>(d_rec), d_pw, n_begin, n_end,
              &rows);
   const size_t row_bytes = sizeof(RowDescF32) * rows.size();
-  // the search for a batch's launch shape marches trials from the state
-  // buffer, so the input goes there first
-  MarchInput from = in;
-  if (spread_lc(plan, steps) == 0 && plan->nb > 1) {
-    rc = copy_input(in, state, st);
-    if (rc != BPM_OK) return rc;
-    from.src = state;
-    from.kind = MarchInput::kC64;
-  }
-  const LaunchShape sh = choose_shape(plan, aux, state, n_begin, steps, st);
+  const LaunchShape sh = choose_shape(plan, aux, in, n_begin, steps, st);
   plan->shape_layout = sh.layout;
   plan->shape_chunk =
       sh.rotated ? std::min(steps, sh.chunk > 0 ? sh.chunk
                                                 : std::max(std::min(steps, 64), steps / 24))
                  : 0;
-  rc = stage_march(plan, aux, from, state, g, rows.data(), sh.rotated ? 0 : row_bytes, st,
-                   captured);
+  rc = stage_march(plan, aux, in, state, g, rows.data(), sh.rotated ? 0 : row_bytes, st, captured);
   if (rc != BPM_OK) return rc;
   if (!sh.rotated) {
     const RowDescF32* d_rows = static_cast<const RowDescF32*>(plan->d_rows);
