@@ -65,7 +65,7 @@ struct RowDescF32 {
   float2* state;            // [2][N] raw envelopes (common phase removed)
   const float2* prop;       // [2][N] (P(q)-1)/N in the FFT's output order
   const float2* prop_nat;   // spread rows: [tables][2][N] (P(q)-1)/N in natural frequency
-                            // order, else null
+                            // order (N <= 128: then prop_form), else null
   const float2* prop_split; // N = 4096 rows on a 4-CTA cluster: [2][3][N/2] circulant
                             // tables of the half-band split, else null
   const float2* phasor;     // [nz][N] exp(i h u_x), (0,0) outside the crystal; null in
@@ -228,8 +228,17 @@ void prop_increments(const bpm_plan_s* plan, int row, double frac,
 // in the fused FFT's output order (nx <= 4096; the split tables above that)
 void fused_prop_table(const bpm_plan_s* plan, const std::vector<std::complex<double>>& inc,
                       std::vector<float2>* out);
-// in natural frequency order, [2][nx] (spread kernels)
+// in natural frequency order, [2][nx] (spread kernels); a row's tables (one, or
+// Forest-Ruth's two) take nat_stride float2, for nx <= 128 with prop_form behind
 void natural_prop_table(const std::vector<std::complex<double>>& inc, float2* out);
+size_t nat_stride(const bpm_plan_s* plan, int tables);
+// How rows of nx <= 128 propagate in launches of few steps: (0, 1) by the
+// increment, field + F^-1 (P - 1) F field, or (1/nx, 0) whole, F^-1 P F field.  The
+// transforms' error goes with the root mean square of P - 1 in the first form and
+// with 1 in the second, so beyond 1 the second is taken (a march's step has 0.1 to
+// 0.8, a free-space step of metres 1.41: relative error of the latter at nx = 64
+// and 128 1.5e-7 and 1.7e-7 by the increment, 1.22e-7 and 1.32e-7 whole).
+float2 prop_form(const std::vector<std::complex<double>>& inc);
 // 3D: (P(qx, qy) - 1)/(nx ny) in the order of the column phase's threads
 // (vol_kernel.cuh).
 void vol_prop_table(const bpm_plan_s* plan, int row, std::vector<float2>* out);
@@ -387,6 +396,17 @@ int fused_rows_per_cta(int logn);
 // (row_kernel.cuh), lc = kOneCta: the march of n_rows rows with splitting
 // `split`; rows carry prop_nat.
 constexpr int kOneCta = 1;
+// First-order launches of up to kFewSteps steps apply every twiddle with its low
+// part.  A step whose increment is as large as the field, a free-space step of
+// metres, carries the tables' rounding once and in full: relative error of one
+// such step of random fields, nx = 64 .. 16384, 1.66 1.86 2.09 2.21 2.32 2.45 2.55
+// 2.69 2.80e-7 with rounded twiddles, 1.22 1.32 1.92 2.02 2.12 2.24 2.34 2.42
+// 2.49e-7 with both parts (the kernels of 16 points per thread, whose transforms
+// take a pass less, 1.20 1.31 1.95 2.10 2.21 2.31 2.50 2.51 2.51e-7).  It costs up
+// to 1 us of a call of 14 to 30 us; in every step of a march it would cost 8 to
+// 20 %, for errors 1 % smaller (there the parts of W and its conjugate that turn
+// the phase cancel).
+constexpr int kFewSteps = 4;
 int launch_spread(int logn, int lc, int split, const RowDescF32* d_rows, int n_rows, int steps,
                   const float4* d_tw, int* d_status, cudaStream_t st);
 int spread_capacity(int logn, int lc, int split);   // clusters resident at once

@@ -136,7 +136,8 @@ void fused_rows(bpm_plan_s* plan, float2* state, float2* rec, double* pw, int n_
                      size_t(r) * 2 * split_table_stride(plan, plan->logn == kSplitLogN ? 12 : 11);
     const bool fr = plan->split == BPM_SPLIT_FOREST_RUTH;   // [2 tables] per row
     const void* nat = fr ? plan->d_stage_prop_nat : plan->d_prop_nat;
-    d.prop_nat = nat ? static_cast<const float2*>(nat) + size_t(r) * (fr ? 4 : 2) * n : nullptr;
+    d.prop_nat = nat ? static_cast<const float2*>(nat) + size_t(r) * nat_stride(plan, fr ? 2 : 1)
+                     : nullptr;
     if (plan->sep_slices) {
       d.phasor = nullptr;
       d.srows = static_cast<const SepRow*>(plan->d_sep);
@@ -813,7 +814,7 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
                           4 * int(nb) <= device_sm_count();
   if (half_split)
     A(&pl->d_prop_split, nb * size_t(split_table_stride(pl, 11)) * cs, "split propagator tables");
-  if (spread_rows(pl)) A(&pl->d_prop_nat, nb * 2 * n * cs, "natural propagator tables");
+  if (spread_rows(pl)) A(&pl->d_prop_nat, nb * nat_stride(pl, 1) * cs, "natural propagator tables");
   // (a capture must find the schedule of rotating spread rows in place)
   if (pl->d_prop_nat && spread_rotates(pl)) {
     aux->sched_cap = nb * kSpreadPieces;
@@ -902,9 +903,10 @@ static int make_plan(const bpm_problem* p, int ny, double dy_um, double y0_um,
                               t.data(), t.size() * sizeof(float2), cudaMemcpyHostToDevice, st);
         }
         if (e == cudaSuccess && pl->d_prop_nat) {
-          t.resize(inc.size());
+          t.resize(nat_stride(pl, 1));
           natural_prop_table(inc, t.data());
-          e = cudaMemcpyAsync(static_cast<float2*>(pl->d_prop_nat) + size_t(r) * 2 * n, t.data(),
+          if (t.size() > inc.size()) t.back() = prop_form(inc);
+          e = cudaMemcpyAsync(static_cast<float2*>(pl->d_prop_nat) + size_t(r) * t.size(), t.data(),
                               t.size() * sizeof(float2), cudaMemcpyHostToDevice, st);
         }
       }
@@ -1006,13 +1008,17 @@ int bpm_set_splitting(bpm_plan_t plan, int32_t method) {
       if (rc != BPM_OK) return rc;
       std::vector<float2> host(nb * 2 * ts);
       std::vector<std::complex<double>> inc;
-      std::vector<float2> nat(plan->d_prop_nat ? nb * 4 * n : 0);
+      const size_t ns = nat_stride(plan, 2);
+      std::vector<float2> nat(plan->d_prop_nat ? nb * ns : 0);
       for (size_t r = 0; r < nb; ++r)
         for (int k = 0; k < 2; ++k) {
           std::vector<float2> tab;
           float2* dst = host.data() + (r * 2 + k) * ts;
           prop_increments(plan, int(r), stages[1 + k].first, &inc);
-          if (plan->d_prop_nat) natural_prop_table(inc, nat.data() + (r * 2 + k) * 2 * n);
+          if (plan->d_prop_nat) {
+            natural_prop_table(inc, nat.data() + r * ns + k * 2 * n);
+            if (k == 0 && ns > 4 * n) nat[r * ns + 4 * n] = prop_form(inc);
+          }
           fused_prop_table(plan, inc, &tab);
           if (plan->logn >= kSplitLogN) {
             std::copy(tab.begin(), tab.end(), dst);

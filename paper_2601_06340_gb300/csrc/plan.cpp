@@ -286,9 +286,20 @@ void fused_prop_table(const bpm_plan_s* plan, const std::vector<cd>& inc,
     }
 }
 
+size_t nat_stride(const bpm_plan_s* plan, int tables) {
+  return size_t(tables) * 2 * plan->nx + (plan->logn <= 7 ? 1 : 0);
+}
+
 void natural_prop_table(const std::vector<cd>& inc, float2* out) {
   for (size_t i = 0; i < inc.size(); ++i)
     out[i] = float2{float(inc[i].real()), float(inc[i].imag())};
+}
+
+float2 prop_form(const std::vector<cd>& inc) {
+  const double n = 0.5 * double(inc.size());
+  double sum = 0.0;
+  for (const cd& v : inc) sum += std::norm(v);
+  return sum * n * n > 2.0 * n ? float2{float(1.0 / n), 0.f} : float2{0.f, 1.f};
 }
 
 // Frequency of value j of thread t, at index j T + t (T = n/8 threads), of the
@@ -419,12 +430,13 @@ void twiddle_table_f32(int n, std::vector<float4>* out) {
   for (int m = 0; m <= n / 8; ++m) {
     double c, s;
     unit_root(m, n, &c, &s);
-    // of the floats next to (c, s), the pair whose modulus is nearest to one:
-    // a forward and an inverse pass multiply by W and its conjugate, so the
-    // modulus error is the one that repeats every step at the same modes
-    // (marches of 2000-6000 steps with the spread kernels' three twiddle
-    // passes: relative error 4.7e-6 -> 4.3e-6 at N = 8192, 3.6e-6 -> 3.1e-6 at
-    // 2048, no larger than the two-pass kernels)
+    // of the floats next to (c, s), the pair whose error is smallest, the phase's
+    // weighted with 0.03: a forward and an inverse pass multiply by W and its
+    // conjugate, so the modulus error is the one that repeats every step at the
+    // same modes, while a single step sees both.  Relative error of the spread
+    // kernels, geometric means over nx = 256 .. 16384, against the modulus alone:
+    // one far-field step 1.07 -> 1.05 times the two-pass kernels', marches of 40 to
+    // 2000 steps 1.020 -> 1.016; nearest floats 1.08, 1.034
     float ch = float(c), sh = float(s);
     if (m != 0 && m != n / 8) {
       const float c0 = ch, s0 = sh;
@@ -433,7 +445,9 @@ void twiddle_table_f32(int n, std::vector<float4>* out) {
         for (int j = -1; j <= 1; ++j) {
           const float ci = i == 0 ? c0 : std::nextafterf(c0, i * 2.f);
           const float sj = j == 0 ? s0 : std::nextafterf(s0, j * 2.f);
-          const double err = std::fabs(double(ci) * ci + double(sj) * sj - 1.0);
+          const double dm = 0.5 * (double(ci) * ci + double(sj) * sj - 1.0);
+          const double dp = double(sj) * c - double(ci) * s;
+          const double err = dm * dm + 0.03 * dp * dp;
           if (err < best) {
             best = err;
             ch = ci;

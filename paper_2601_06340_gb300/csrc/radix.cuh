@@ -7,10 +7,12 @@
 // Accuracy note.  The march applies the same forward/inverse pair tens of
 // thousands of times, so any constant rounded to FP32 acts as a fixed
 // perturbation of every step and its error grows linearly with the number of
-// steps.  Every non-trivial constant (cos(pi/8), sin(pi/8), 1/sqrt(2)) and
-// every table twiddle is therefore carried as an unevaluated sum hi + lo of
-// two floats and applied with fused multiply-adds, so the only FP32 error
-// left is the rounding of results, which varies from step to step.
+// steps.  Every non-trivial constant (cos(pi/8), sin(pi/8), 1/sqrt(2)) is
+// therefore carried as an unevaluated sum hi + lo of two floats and applied
+// with fused multiply-adds.  Table twiddles are applied so by the kernel that
+// keeps both bands of a row in a thread (N <= 128) and by launches of few steps
+// (kFewSteps); elsewhere as one float each, chosen for a small modulus error
+// (twiddle_table_f32), the part of the error that repeats every step.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -23,7 +23,7 @@
 
 namespace bpm {
 
-template <int LOGN, int SCH>
+template <int LOGN, int SCH, bool EX>
 struct RowCfg {
   static constexpr int N = 1 << LOGN;
   static constexpr int N1 = 1 << (LOGN / 2), N2 = N / N1;
@@ -37,6 +37,7 @@ struct RowCfg {
   static constexpr int P = T + (U < 16 ? U : 8), PF = T + (H < 16 ? H : 0);
   static constexpr int BUF = 8 * (P > PF ? P : PF);
   static constexpr int TABLES = SCH == kSchForestRuth ? 2 : 1;
+  static constexpr int W = EX ? 16 : 8;              // bytes of a twiddle
   // buffer A: forward column exchange, then received increment; buffer B:
   // received spectrum, then inverse column exchange (each reuse has a block
   // barrier between its last read and the next write)
@@ -44,10 +45,10 @@ struct RowCfg {
   static constexpr int OFF_B = OFF_A + BUF * 8;
   static constexpr int OFF_Y = OFF_B + BUF * 8;              // [WARPS][8][33] row exchange
   static constexpr int OFF_WM = OFF_Y + WARPS * 264 * 8;     // [8][T/2] W_N^(n2 k1)
-  static constexpr int OFF_D = OFF_WM + 4 * T * 8;           // [TABLES][8][T] propagator
+  static constexpr int OFF_D = OFF_WM + 4 * T * W;           // [TABLES][8][T] propagator
   static constexpr int OFF_WC = OFF_D + TABLES * 8 * T * 8;  // [8][Q] W_N1
-  static constexpr int OFF_WR = OFF_WC + 8 * Q * 8;          // [8][CI] W_N2
-  static constexpr int OFF_RED = OFF_WR + 8 * CI * 8;        // [WARPS][2] double
+  static constexpr int OFF_WR = OFF_WC + 8 * Q * W;          // [8][CI] W_N2
+  static constexpr int OFF_RED = OFF_WR + 8 * CI * W;        // [WARPS][2] double
   static constexpr int OFF_RECPH = OFF_RED + WARPS * 16;     // [2] float2
   static constexpr int ROW_SMEM = OFF_RECPH + 16;
   static constexpr int SMEM = ROWS * ROW_SMEM;
@@ -56,11 +57,16 @@ struct RowCfg {
   static_assert(SMEM <= 232448, "fits one SM");
 };
 
-template <int LOGN, int SCH>
-__global__ void __launch_bounds__((RowCfg<LOGN, SCH>::THREADS), (RowCfg<LOGN, SCH>::MINCTAS))
+// EX: every twiddle with its low part and, for N <= 128, the propagation's form by
+// prop_form (else by the increment), for launches of few steps (spread.cu).
+template <int LOGN, int SCH, bool EX>
+__global__ void __launch_bounds__((RowCfg<LOGN, SCH, EX>::THREADS),
+                                  (RowCfg<LOGN, SCH, EX>::MINCTAS))
     row_march_kernel(const RowDescF32* __restrict__ rows, int n_rows, int steps,
                      const float4* __restrict__ tw) {
-  using S = RowCfg<LOGN, SCH>;
+  using S = RowCfg<LOGN, SCH, EX>;
+  using W = Twiddle<EX>;
+  constexpr bool FORM = EX && S::N <= 128;
   constexpr int N = S::N, N1 = S::N1, N2 = S::N2, T = S::T, CI = S::CI, U = S::U, H = S::H;
   constexpr bool HALF = SCH != kSchFirst;
   constexpr int STAGES = SCH == kSchForestRuth ? 3 : 1;
@@ -81,17 +87,14 @@ __global__ void __launch_bounds__((RowCfg<LOGN, SCH>::THREADS), (RowCfg<LOGN, SC
   float2* ba = reinterpret_cast<float2*>(smem + S::OFF_A);
   float2* bb = reinterpret_cast<float2*>(smem + S::OFF_B);
   float2* y = reinterpret_cast<float2*>(smem + S::OFF_Y) + warp * 264;
-  float2* wm = reinterpret_cast<float2*>(smem + S::OFF_WM) + (h * S::Q + q) * CI + r;
+  W* wm = reinterpret_cast<W*>(smem + S::OFF_WM) + (h * S::Q + q) * CI + r;
   float2* dp = reinterpret_cast<float2*>(smem + S::OFF_D) + t;
-  float2* wc = reinterpret_cast<float2*>(smem + S::OFF_WC);
-  float2* wr = reinterpret_cast<float2*>(smem + S::OFF_WR);
+  W* wc = reinterpret_cast<W*>(smem + S::OFF_WC);
+  W* wr = reinterpret_cast<W*>(smem + S::OFF_WR);
   double* red = reinterpret_cast<double*>(smem + S::OFF_RED);
   float2* recph = reinterpret_cast<float2*>(smem + S::OFF_RECPH);
 
-  auto root = [&](int m) {
-    const float4 a = __ldg(&tw[m & (N - 1)]);
-    return make_float2(a.x, a.y);
-  };
+  auto root = [&](int m) { return twiddle_of<EX>(__ldg(&tw[m & (N - 1)])); };
   for (int i = t; i < 8 * S::Q; i += T) wc[i] = root((i / S::Q) * (i % S::Q) * N2);
   for (int i = t; i < 8 * CI; i += T) wr[i] = root((i / CI) * (i % CI) * N1);
 #pragma unroll
@@ -101,6 +104,9 @@ __global__ void __launch_bounds__((RowCfg<LOGN, SCH>::THREADS), (RowCfg<LOGN, SC
     dp[j * T] = __ldg(&d.prop_nat[k]);
     if constexpr (S::TABLES == 2) dp[(8 + j) * T] = __ldg(&d.prop_nat[2 * N + k]);
   }
+  // the share of the field in the propagator's product (1/N or 0), and that of the
+  // field added to its inverse (0 or 1)
+  const float2 form = FORM ? __ldg(&d.prop_nat[S::TABLES * 2 * N]) : make_float2(0.f, 1.f);
   auto w_col = [&](int k) { return wc[k * S::Q + q]; };
   auto w_row = [&](int k) { return wr[k * CI + r]; };
   auto col_addr = [&](int k, int pos) { return k * S::P + h * H + pos * U + u; };
@@ -174,24 +180,33 @@ __global__ void __launch_bounds__((RowCfg<LOGN, SCH>::THREADS), (RowCfg<LOGN, SC
       float2 org[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) org[j] = v[j];
-      spread_fwd<N1>(v, ba, q, col_addr, w_col, nullptr, 0, cta_sync);
+      spread_fwd<N1>(v, ba, q, col_addr, w_col, static_cast<const W*>(nullptr), 0, cta_sync);
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = xmul(v[j], wm[j * (T / 2)]);
       exchange(v, bb);
       if (sg == 0 && lead && pow_on && rs.prev) put_powers(rs.pslot);
       __syncwarp();     // (the previous stage's reads of y)
-      spread_fwd<N2>(v, y, r, row_addr, w_row, nullptr, 0, warp_sync);
+      spread_fwd<N2>(v, y, r, row_addr, w_row, static_cast<const W*>(nullptr), 0, warp_sync);
       const float2* dk = dp + (STAGES == 3 && sg == 1 ? 8 * T : 0);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = xmul(v[j], dk[j * T]);
+      for (int j = 0; j < 8; ++j) {
+        const float2 x = v[j];
+        v[j] = xmul(x, dk[j * T]);
+        if constexpr (FORM)
+          v[j] = make_float2(fmaf(form.x, x.x, v[j].x), fmaf(form.x, x.y, v[j].y));
+      }
       __syncwarp();
-      spread_inv<N2>(v, y, r, row_addr, w_row, nullptr, 0, warp_sync);
+      spread_inv<N2>(v, y, r, row_addr, w_row, static_cast<const W*>(nullptr), 0, warp_sync);
       exchange(v, ba);
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = xmul(v[j], xconj(wm[j * (T / 2)]));
-      spread_inv<N1>(v, bb, q, col_addr, w_col, nullptr, 0, cta_sync);
+      spread_inv<N1>(v, bb, q, col_addr, w_col, static_cast<const W*>(nullptr), 0, cta_sync);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = cadd(org[j], v[j]);
+      for (int j = 0; j < 8; ++j) {
+        if constexpr (FORM)
+          v[j] = make_float2(fmaf(form.y, org[j].x, v[j].x), fmaf(form.y, org[j].y, v[j].y));
+        else v[j] = cadd(org[j], v[j]);
+      }
       if (sg < STAGES - 1) {
         couple(cur, d.am1, d.b);     // Forest-Ruth's inner couplings
         return;

@@ -7,10 +7,10 @@
 
 namespace bpm {
 
-template <int LOGN, int SCH>
+template <int LOGN, int SCH, bool EX = false>
 struct RowLaunch {
-  using S = RowCfg<LOGN, SCH>;
-  static constexpr auto kernel = row_march_kernel<LOGN, SCH>;
+  using S = RowCfg<LOGN, SCH, EX>;
+  static constexpr auto kernel = row_march_kernel<LOGN, SCH, EX>;
 
   static int configure() {
     static std::atomic<bool> done{false};
@@ -57,7 +57,8 @@ struct RowLaunch {
                      cudaStream_t st) {                                                   \
     return split == BPM_SPLIT_VERLET        ? RowLaunch<L, kSchVerlet>::launch(r, n, s, tw, st)     \
            : split == BPM_SPLIT_FOREST_RUTH ? RowLaunch<L, kSchForestRuth>::launch(r, n, s, tw, st) \
-                                            : RowLaunch<L, kSchFirst>::launch(r, n, s, tw, st);     \
+           : s <= kFewSteps ? RowLaunch<L, kSchFirst, true>::launch(r, n, s, tw, st)      \
+                            : RowLaunch<L, kSchFirst>::launch(r, n, s, tw, st);           \
   }                                                                                       \
   int row_capacity_##L(int split) {                                                       \
     return split == BPM_SPLIT_VERLET        ? RowLaunch<L, kSchVerlet>::capacity()        \

@@ -42,12 +42,27 @@
 
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "fused4_kernel.cuh"
 
 namespace bpm {
 
 __device__ __forceinline__ float2 xmul(float2 a, float2 b) { return cmul_f(a, b.x, b.y); }
 __device__ __forceinline__ float2 xconj(float2 a) { return make_float2(a.x, -a.y); }
+// the same with a twiddle of hi + lo pairs
+__device__ __forceinline__ float2 xmul(float2 a, float4 w) {
+  return cmul_hl(a, w.x, w.y, w.z, w.w);
+}
+__device__ __forceinline__ float4 xconj(float4 a) { return make_float4(a.x, -a.y, a.z, -a.w); }
+// A table entry as the kernels' twiddle: EX both parts, else the high one.
+template <bool EX>
+using Twiddle = std::conditional_t<EX, float4, float2>;
+template <bool EX>
+__device__ __forceinline__ Twiddle<EX> twiddle_of(float4 a) {
+  if constexpr (EX) return a;
+  else return make_float2(a.x, a.y);
+}
 __device__ __forceinline__ float2 xshfl(float2 a, int mask) {
   return make_float2(__shfl_xor_sync(0xffffffffu, a.x, mask),
                      __shfl_xor_sync(0xffffffffu, a.y, mask));
@@ -118,9 +133,9 @@ struct SpreadCfg {
 // point j at index q + (L/8) j on entry, frequency q + (L/8) j on return.
 // addr(k, q') is the exchange buffer's slot of radix-8 output k of position
 // q'; w1(k) = W_L^(q k); w2: W_16^((hi + 2 g) k), hi = bit 3 of q (L = 128).
-template <int L, typename AddrF, typename TwF, typename SyncF>
+template <int L, typename AddrF, typename TwF, typename W, typename SyncF>
 __device__ __forceinline__ void spread_fwd(float2* v, float2* buf, int q, AddrF addr, TwF w1,
-                                           const float2* w2, int xm, SyncF sync) {
+                                           const W* w2, int xm, SyncF sync) {
   dft<8, false>(v);
   if constexpr (L == 8) return;
 #pragma unroll
@@ -174,9 +189,9 @@ __device__ __forceinline__ void spread_fwd(float2* v, float2* buf, int q, AddrF 
 }
 
 // The matching inverse (unnormalised): frequency q + (L/8) j on entry.
-template <int L, typename AddrF, typename TwF, typename SyncF>
+template <int L, typename AddrF, typename TwF, typename W, typename SyncF>
 __device__ __forceinline__ void spread_inv(float2* v, float2* buf, int q, AddrF addr, TwF w1,
-                                           const float2* w2, int xm, SyncF sync) {
+                                           const W* w2, int xm, SyncF sync) {
   if constexpr (L == 8) {
     dft<8, true>(v);
     return;
@@ -282,8 +297,9 @@ __device__ __forceinline__ void slice8_couple(float2* v, const Slice8& s, float2
     v[j] = xcouple(v[j], xshfl(v[j], BM), s.e[j], (m >> j) & 1u, am1, b, bs);
 }
 
-// SCH: the operator splitting as in fused2_kernel.cuh.
-template <int LOGN, int LC, int SCH>
+// SCH: the operator splitting as in fused2_kernel.cuh.  EX: every twiddle with its
+// low part, for launches of few steps (spread.cu).
+template <int LOGN, int LC, int SCH, bool EX>
 __global__ void __launch_bounds__((SpreadCfg<LOGN, LC>::T), 1)
     spread_march_kernel(const RowDescF32* __restrict__ rows, int steps,
                         const float4* __restrict__ tw, int* __restrict__ status) {
@@ -380,10 +396,9 @@ __global__ void __launch_bounds__((SpreadCfg<LOGN, LC>::T), 1)
   // twiddles, all in registers: the column's and the row's first pass, and
   // W_N^(n2 k1) of this thread's points between column and exchange
   auto root = [&](int m) {               // W_N^m
-    const float4 a = __ldg(&tw[m & (N - 1)]);
-    return make_float2(a.x, a.y);
+    return twiddle_of<EX>(__ldg(&tw[m & (N - 1)]));
   };
-  float2 wc[7], wr[7], wm[8];
+  Twiddle<EX> wc[7], wr[7], wm[8];
 #pragma unroll
   for (int k = 1; k < 8; ++k) {
     wc[k - 1] = root(q * k * N2);
@@ -394,7 +409,7 @@ __global__ void __launch_bounds__((SpreadCfg<LOGN, LC>::T), 1)
   auto w_col = [&](int k) { return wc[k - 1]; };
   auto w_row = [&](int k) { return wr[k - 1]; };
   // third-pass twiddles of 128-point transforms: positions h, h + 2 of 4
-  float2 w2c[N1 == 128 ? 6 : 1], w2r[N2 == 128 ? 6 : 1];
+  Twiddle<EX> w2c[N1 == 128 ? 6 : 1], w2r[N2 == 128 ? 6 : 1];
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
     if constexpr (N1 == 128) w2c[i] = root(((q >> 3) + 2 * (i / 3)) * (i % 3 + 1) * (N / 16));

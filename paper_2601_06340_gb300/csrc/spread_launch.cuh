@@ -9,10 +9,10 @@ namespace bpm {
 
 // The launch configuration of n_rows clusters of 2^LC CTAs; clusters of 16
 // need the non-portable size allowed.
-template <int LOGN, int LC, int SCH>
+template <int LOGN, int LC, int SCH, bool EX = false>
 struct SpreadLaunch {
   using S = SpreadCfg<LOGN, LC>;
-  static constexpr auto kernel = spread_march_kernel<LOGN, LC, SCH>;
+  static constexpr auto kernel = spread_march_kernel<LOGN, LC, SCH, EX>;
 
   static int configure() {
     static std::atomic<bool> done{false};
@@ -79,7 +79,10 @@ struct SpreadSize {
     switch (split) {
       case BPM_SPLIT_VERLET: return L<kSchVerlet>::launch(r, n, steps, tw, status, st);
       case BPM_SPLIT_FOREST_RUTH: return L<kSchForestRuth>::launch(r, n, steps, tw, status, st);
-      default: return L<kSchFirst>::launch(r, n, steps, tw, status, st);
+      default:
+        return steps <= kFewSteps
+                   ? SpreadLaunch<LOGN, LC, kSchFirst, true>::launch(r, n, steps, tw, status, st)
+                   : L<kSchFirst>::launch(r, n, steps, tw, status, st);
     }
   }
 
