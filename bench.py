@@ -42,9 +42,12 @@ WORKLOAD = ("bragg_bent: 2D symmetric Bragg, bent crystal R=1 m nu=0.28, 8 keV, 
             "theta_B=23.65 deg, 200 um slab, Nx=4096, Nz=8000, dx=0.2 um, dz=0.1 um, "
             "one energy, Gaussian 50 um FWHM")
 FLOPS_PER_CELL = lambda n: 4 * 5 * math.log2(n)      # 4 FFTs x 5 N log2 N / N
-# the single-solve march kernel by launch layout (bpm_launch_shape): name, SMs
+# the single-solve march kernel by launch layout (bpm_launch_shape; "spread": rows on
+# clusters of 8 or 16 CTAs, bpm_launch_ctas): name, SMs
 MARCH_KERNELS = {
-    2: ("spread_march_kernel<12, 4> (16-CTA cluster per solve, 8 points per thread)", 16),
+    "spread": ("spread_march_kernel<12, 4> (16-CTA cluster per solve, 8 points per thread)", 16),
+    2: ("fused4s_march_kernel (4-CTA cluster per solve: two half-band parts per band, "
+        "8 points per thread)", 4),
     8: ("fused4e_march_kernel<11> (4-CTA cluster per solve: two half-band parts per band, "
         "16 points per thread)", 4),
     1: ("fused3_march_kernel<12> (2-CTA cluster per solve, one band per CTA)", 2),
@@ -677,6 +680,8 @@ def run_gpu(args, rks):
     value = world * args.steps * cells / (total_ms * 1e-3)
     clocks = clk.summary()
     march_layout, _ = binding.bpm_launch_shape(plan32.handle)
+    if binding.bpm_launch_ctas(plan32.handle) > 1:
+        march_layout = "spread"
 
     if args.only == "fused":
         if rank == 0:

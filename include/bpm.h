@@ -356,7 +356,9 @@ int bpm_march_f64_noalloc(void* d_psi, int32_t nx, int32_t n_rows, const void* d
  * spread over clusters of 8 or 16 CTAs else (nx = 1024 to 136 rows; 2048 from
  * 72 rows, 4096 from 36, 8192 from 15, 16384 from 7 on in rotation, up to about
  * 1.5 times these rows, or more where the other forms need further waves);
- * they report the code below that their size and splitting had as single rows.  *layout = 10
+ * bpm_launch_ctas tells them; here they report the code that their size and splitting
+ * had as single rows before (first-order batches of 512 to 2048: the fixed rule's -1 where
+ * the search below is switched off, else 2, or 0 on one CTA).  *layout = 10
  * the Forest-Ruth step on one cluster per row (512 <= nx <= 4096), 9 the
  * Forest-Ruth step on one cluster per row (nx = 4096 and 8192: 4-CTA
  * half-band split, split band), 8 the nx = 4096 half-band split with 16
@@ -381,6 +383,13 @@ int bpm_march_f64_noalloc(void* d_psi, int32_t nx, int32_t n_rows, const void* d
  * row leaves the fixed rule in charge.  Either
  * pointer may be NULL.  BPM_ERR_INVALID for a NULL plan. */
 int bpm_launch_shape(bpm_plan_t plan, int32_t* layout, int32_t* chunk);
+
+/* Kernel family of the plan's last FP32 march in 2D: *ctas = 8 or 16 rows spread
+ * over clusters of as many CTAs, 1 one CTA per row with 8 points per thread (both
+ * report the codes of bpm_launch_shape that their sizes had before), 0 the
+ * kernel that the code of bpm_launch_shape names, or no march yet.
+ * BPM_ERR_INVALID for NULL pointers. */
+int bpm_launch_ctas(bpm_plan_t plan, int32_t* ctas);
 
 /* Release the plan and its device memory.  BPM_ERR_BUSY while tickets of
  * the plan are pending. */

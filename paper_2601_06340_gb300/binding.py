@@ -70,6 +70,7 @@ _SIGS = {
     "bpm_fetch_slices": ([_P, _P, _P], ctypes.c_int),
     "bpm_march_f64_noalloc": ([_P, _I, _I, _P, _P, _P, _I, _I, _P], ctypes.c_int),
     "bpm_launch_shape": ([_P, ctypes.POINTER(_I), ctypes.POINTER(_I)], ctypes.c_int),
+    "bpm_launch_ctas": ([_P, ctypes.POINTER(_I)], ctypes.c_int),
     "bpm_slice_form": ([_P, ctypes.POINTER(_I), ctypes.POINTER(ctypes.c_int64)], ctypes.c_int),
     "bpm_destroy": ([_P], ctypes.c_int),
     "bpm_last_error": ([], ctypes.c_char_p),
@@ -221,7 +222,9 @@ def bpm_march_f64_noalloc(d_psi, nx, n_rows, d_prop, d_coupling, d_phasor, n_beg
 
 
 def bpm_launch_shape(plan) -> tuple[int, int]:
-    """(layout, chunk) of the plan's last FP32 march: layout 10 the
+    """(layout, chunk) of the plan's last FP32 march (rows on the kernels of 8
+    points per thread, see bpm_launch_ctas, report the layout that their size
+    and splitting had before): layout 10 the
     Forest-Ruth step on a two-CTA cluster per row (N = 512-4096), 9 the
     Forest-Ruth step on the N = 4096 half-band split or the N = 8192 split
     band, 8 the 16-point form of the N = 4096 split (forced), 7 the
@@ -234,6 +237,15 @@ def bpm_launch_shape(plan) -> tuple[int, int]:
     layout, chunk = _I(0), _I(0)
     _check(load().bpm_launch_shape(plan, ctypes.byref(layout), ctypes.byref(chunk)))
     return layout.value, chunk.value
+
+
+def bpm_launch_ctas(plan) -> int:
+    """CTAs per row of the plan's last FP32 march on the kernels of 8 points per
+    thread: 8 or 16 a cluster per row, 1 one CTA per row; 0 the kernel that
+    bpm_launch_shape's layout names."""
+    ctas = _I(0)
+    _check(load().bpm_launch_ctas(plan, ctypes.byref(ctas)))
+    return ctas.value
 
 
 def bpm_slice_form(plan) -> tuple[int, int]:

@@ -204,7 +204,7 @@ struct bpm_plan_s {
   int pending = 0;                // tickets not yet finished
   // launch shape of the last fused march: layout 1 cluster / 0 CTA / -1 rule,
   // rotation chunk (0: one launch)
-  int shape_layout = -1, shape_chunk = 0;
+  int shape_layout = -1, shape_chunk = 0, shape_spread = 0;
   bpm::PlanAux aux;
 };
 

@@ -619,6 +619,7 @@ static int march_staged_fr(bpm_plan_s* plan, PlanAux* aux, void* state, void* d_
   }
   plan->shape_layout = kLayoutStagedFR;
   plan->shape_chunk = 0;
+  plan->shape_spread = 0;
   const float4* tw = static_cast<const float4*>(plan->d_tw);
   std::vector<RowDescF32> sched(cap);
   int rc = BPM_OK;
@@ -729,6 +730,7 @@ static int enqueue_march(bpm_plan_s* plan, PlanAux* aux, const MarchInput& in, v
   const size_t row_bytes = sizeof(RowDescF32) * rows.size();
   const LaunchShape sh = choose_shape(plan, aux, in, n_begin, steps, st);
   plan->shape_layout = sh.layout;
+  plan->shape_spread = sh.spread == 0 ? 0 : sh.spread == kOneCta ? 1 : 1 << sh.spread;
   plan->shape_chunk =
       sh.rotated ? std::min(steps, sh.chunk > 0 ? sh.chunk
                                                 : std::max(std::min(steps, 64), steps / 24))
@@ -1463,6 +1465,13 @@ int bpm_launch_shape(bpm_plan_t plan, int32_t* layout, int32_t* chunk) {
   std::lock_guard<std::mutex> lk(plan->mu);
   if (layout) *layout = plan->shape_layout;
   if (chunk) *chunk = plan->shape_chunk;
+  return BPM_OK;
+}
+
+int bpm_launch_ctas(bpm_plan_t plan, int32_t* ctas) {
+  if (!plan || !ctas) return fail(BPM_ERR_INVALID, "plan / ctas is NULL");
+  std::lock_guard<std::mutex> lk(plan->mu);
+  *ctas = plan->shape_spread;
   return BPM_OK;
 }
 
