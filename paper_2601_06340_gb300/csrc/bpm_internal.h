@@ -411,6 +411,13 @@ int launch_spread(int logn, int lc, int split, const RowDescF32* d_rows, int n_r
                   const float4* d_tw, int* d_status, cudaStream_t st);
 int spread_capacity(int logn, int lc, int split);   // clusters resident at once
 int spread_choice(int logn, int rows, int split);   // lc of a launch, 0: not spread
+// Whether the environment keeps rows on the kernels of 16 points per thread:
+// BPM_FUSED_LAYOUT set (read at every march), or plain butterfly constants asked
+// for, which only those have.
+bool forced_16();
+// Butterfly constants as hi + lo pairs (default), or plain floats with
+// BPM_FUSED_EXACT=0 (read once; 2D rows of nx >= 256).
+bool fused_exact_constants();
 // how many steps of a full launch of spread rows the other form's step takes
 double spread_limit(int logn, int rows, int split);
 int fused_threads(int logn);

@@ -376,10 +376,10 @@ static int spread_chunk(int rows, int cap, int steps, double* cost) {
   return best;
 }
 
-// log2 of the CTAs that each row of a plan is spread over, 0 if not (any
-// BPM_FUSED_LAYOUT forces the other forms), and the chunk if they rotate.
+// log2 of the CTAs that each row of a plan is spread over, 0 if not, and the
+// chunk if they rotate.
 static int spread_lc(const bpm_plan_s* plan, int steps, int* chunk = nullptr) {
-  if (!plan->d_prop_nat || std::getenv("BPM_FUSED_LAYOUT")) return 0;
+  if (!plan->d_prop_nat || forced_16()) return 0;
   const int lc = spread_choice(plan->logn, plan->nb, plan->split);
   const int cap = lc > kOneCta ? spread_capacity(plan->logn, lc, plan->split) : 0;
   if (cap > 0 && plan->nb > cap) {

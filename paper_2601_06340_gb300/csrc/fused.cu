@@ -77,6 +77,19 @@ int fused2_rows_resident_12();
 // (read at every launch).
 static int sm_count();
 
+bool fused_exact_constants() {
+  static std::atomic<int> cached{-1};
+  int v = cached.load(std::memory_order_relaxed);
+  if (v < 0) {
+    const char* e = std::getenv("BPM_FUSED_EXACT");
+    v = (e && e[0] == '0') ? 0 : 1;
+    cached.store(v, std::memory_order_relaxed);
+  }
+  return v == 1;
+}
+
+bool forced_16() { return std::getenv("BPM_FUSED_LAYOUT") || !fused_exact_constants(); }
+
 static int forced_layout() {
   const char* v = std::getenv("BPM_FUSED_LAYOUT");
   if (!v) return -1;

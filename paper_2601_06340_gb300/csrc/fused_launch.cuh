@@ -14,18 +14,6 @@
 
 namespace bpm {
 
-// Butterfly-constant policy: hi+lo constants (default) unless BPM_FUSED_EXACT=0.
-inline bool fused_exact_constants() {
-  static std::atomic<int> cached{-1};
-  int v = cached.load(std::memory_order_relaxed);
-  if (v < 0) {
-    const char* e = std::getenv("BPM_FUSED_EXACT");
-    v = (e && e[0] == '0') ? 0 : 1;
-    cached.store(v, std::memory_order_relaxed);
-  }
-  return v == 1;
-}
-
 // Both-bands-per-thread kernel (N <= 128); SCH the operator splitting.
 template <int LOGN, int SCH = 0>
 int fused_launch_impl(const RowDescF32* d_rows, int n_rows, int steps,

@@ -435,7 +435,7 @@ int launch_batch(Server& s, Bucket& b) {
   // always one CTA of 8 points per thread, N = 1024 beyond that (2 rows per SM
   // in 3.4 us either way, one in 2.0 against 3.4).
   int spread = 0;
-  if (fp32 && !std::getenv("BPM_FUSED_LAYOUT") && (logn <= 10 || logn >= kSplitLogN ||
+  if (fp32 && !forced_16() && (logn <= 10 || logn >= kSplitLogN ||
                                                    spread_demand(s) <= s.sm_count)) {
     int rows = 0;
     bool tables = true;

@@ -13,6 +13,10 @@ Tolerance: as in test_spread_gpu.py, 40 steps of one rounding of the field each
 2^-24 * sqrt(2 log2 nx) = 1.34e-7 a step: 40 of them, 5.4e-6.
 """
 
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -75,3 +79,21 @@ def test_former_kernels_match_oracle(bpm_lib, monkeypatch, form, split, sizes):
         errs = band_errors(out.psi, ref.psi, out.records, ref.records)
         assert max(errs) <= tol, (nx, errs)
         assert np.allclose(out.powers, ref.powers, rtol=1e-5), nx
+
+
+def test_plain_constants_keep_their_kernels(bpm_lib):
+    """BPM_FUSED_EXACT=0 (read once in a process) asks for plain butterfly constants,
+    which only the kernels of 16 points per thread and the half-band split have."""
+    code = """
+import os
+os.environ.pop("BPM_FUSED_LAYOUT", None)
+from paper_2601_06340_gb300 import binding, inputs
+with binding.Plan(inputs.bragg_bent(nx=1024, nz=8, record_every=0)) as plan:
+    plan.propagate(records=False)
+    print(binding.bpm_launch_ctas(plan.handle))
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    for exact, ctas in (("0", "0"), ("1", "8")):
+        out = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True,
+                             env=dict(os.environ, BPM_FUSED_EXACT=exact), timeout=300)
+        assert out.returncode == 0 and out.stdout.split() == [ctas], (exact, out)
