@@ -401,7 +401,7 @@ const char* bpm_last_error(void);
 /* Library version string. */
 const char* bpm_version(void);
 
-/* Self-test of the bounded device wait that every march kernel uses on its
+/* Self-test of the bounded device wait that the 2D FP32 march kernels use on their
  * mbarriers (strain-slice copies, peer data).  No counterpart in the paper.
  * One CTA arms a barrier for bytes that no copy delivers and waits with the
  * march kernels' bounded loop, which gives up without any fault; the kernel
@@ -411,6 +411,12 @@ const char* bpm_version(void);
  * the kernel ends.  BPM_ERR_INVALID for NULL pointers, BPM_ERR_CUDA if the
  * launch failed. */
 int bpm_selftest_wait_expiry(int32_t* status, double* seconds);
+
+/* The same for the grid barrier of the FP64 and 3D marches: one CTA waits at it
+ * for an arrival that never comes, with a limit of some 4 ms (a march's: 1 s at most,
+ * and 14 to 40 s for its first barrier, at which CTAs may still have to wait for other
+ * kernels to leave their SMs), and does not wait at the next one. */
+int bpm_selftest_barrier_expiry(int32_t* status, double* seconds);
 
 /* Measured arithmetic peak of the current device: the denominator of the
  * march kernels' roofline fractions (the march is bound by FP32 ALU work;

@@ -76,6 +76,8 @@ _SIGS = {
     "bpm_last_error": ([], ctypes.c_char_p),
     "bpm_version": ([], ctypes.c_char_p),
     "bpm_selftest_wait_expiry": ([ctypes.POINTER(_I), ctypes.POINTER(ctypes.c_double)], ctypes.c_int),
+    "bpm_selftest_barrier_expiry": ([ctypes.POINTER(_I), ctypes.POINTER(ctypes.c_double)],
+                                    ctypes.c_int),
     "bpm_server_inject_launch_failure": ([_I, _I], ctypes.c_int),
     "bpm_device_status": ([_P, _P], ctypes.c_int),
     "bpm_fp_peak": ([_I, _I, ctypes.POINTER(_D), ctypes.POINTER(_D)], ctypes.c_int),
@@ -266,6 +268,14 @@ def bpm_selftest_wait_expiry() -> tuple[int, float]:
 
 
 BPM_PEAK_FP64_DFMA, BPM_PEAK_FP32_FFMA, BPM_PEAK_FP32_FFMA2 = 0, 1, 2
+
+
+def bpm_selftest_barrier_expiry() -> tuple[int, float]:
+    """(status, seconds): one CTA waits at the FP64 and 3D marches' grid barrier
+    for an arrival that never comes; status 1 means that the wait expired."""
+    status, seconds = _I(0), ctypes.c_double(0.0)
+    _check(load().bpm_selftest_barrier_expiry(ctypes.byref(status), ctypes.byref(seconds)))
+    return status.value, seconds.value
 
 
 def bpm_fp_peak(kind: int, iters: int) -> tuple[float, float]:
