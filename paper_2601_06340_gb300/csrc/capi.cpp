@@ -224,20 +224,22 @@ static int launch_rotated(bpm_plan_s* plan, PlanAux* aux, const std::vector<RowD
   chunk = std::min(chunk, steps);
   const int full = steps / chunk, rem = steps - full * chunk;
   std::vector<RowDescF32> sched;
-  struct Launch { size_t off; int count; int steps; };
+  struct Launch { size_t off; int count; int steps; bool mixed; };
   std::vector<Launch> launches;
   auto round = [&](int c0, int c1) {
     const long items = long(nb) * (c1 - c0);
     for (long i = 0; i < items; i += resident) {
       const int cnt = int(std::min<long>(resident, items - i));
-      launches.push_back({sched.size(), cnt, 0});
+      launches.push_back({sched.size(), cnt, 0, false});
       for (int k = 0; k < cnt; ++k) {
         const long it = i + k;
         RowDescF32 d = rows[it % nb];
         const int at = int(c0 + it / nb) * chunk, len = std::min(chunk, steps - at);
         d.n_begin = n_begin + at;
         d.n_end = d.n_begin + len;
-        launches.back().steps = std::max(launches.back().steps, len);
+        Launch& l = launches.back();
+        l.mixed = l.mixed || (k > 0 && len != l.steps);
+        l.steps = std::max(l.steps, len);
         sched.push_back(d);
       }
     }
@@ -268,10 +270,16 @@ static int launch_rotated(bpm_plan_s* plan, PlanAux* aux, const std::vector<RowD
   for (const Launch& l : launches) {
     const RowDescF32* d_rows = aux->d_sched + l.off;
     const float4* tw = static_cast<const float4*>(plan->d_tw);
+    // Items of different lengths in one launch need a kernel that stops at its
+    // row's last step: the spread kernel, or one CTA per row (layout 0, 3, 6).
+    // The rule (-1) may take the 2-CTA cluster, which does not, for a short tail;
+    // one CTA is forced there (a tail of at most nb items, all of the rows' last
+    // chunks, is not mixed).
+    const int lay = l.mixed && layout < 0 ? 0 : layout;
     int rc = spread ? launch_spread(plan->logn, spread, plan->split, d_rows, l.count, l.steps, tw,
                                     plan->d_status, st)
                     : launch_fused_layout(plan->logn, d_rows, l.count, l.steps, tw,
-                                          plan->d_status, st, layout);
+                                          plan->d_status, st, lay);
     if (rc != BPM_OK) return rc;
   }
   return BPM_OK;

@@ -10,9 +10,9 @@ namespace bpm {
 // by its distance from the target, so it may wrap), with a bounded wait: `later`
 // polls of 0.2 us (one CTA) to about 0.6 us (all SMs polling), one second at most,
 // and `first` polls, 14 to 40 seconds, for the launch's first barrier, which may
-// have to wait for other kernels to leave the SMs that the last CTAs need.  After an expired wait the CTA raises and waits no
-// more, so the others' waits expire too and the launch ends.  1.13 us on GB300
-// between 8 to 152 CTAs.
+// have to wait for other kernels to leave the SMs that the last CTAs need.  After
+// an expired wait the CTA raises and waits no more, so the others' waits expire
+// too and the launch ends.  1.13 us on GB300 between 8 to 152 CTAs.
 struct GridBarrier {
   unsigned* counter;
   int* s_dead;                // shared: a wait of this CTA expired
