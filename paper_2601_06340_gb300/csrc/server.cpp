@@ -428,12 +428,13 @@ int launch_batch(Server& s, Bucket& b) {
     for (auto& r : b.members) tables = tables && r->plan->d_prop_split != nullptr;
     if (tables) layout = kLayoutSplit4;
   }
-  // First-order rows spread over clusters of up to 16 SMs: N >= 8192 always
-  // (a row's SM time is no more than on the split bands: 8192 24 against 22
-  // SM us per step at full load, 16384 71 against 78, and its latency half),
-  // N = 1024 to 4096 while the whole active set fits the GPU that way; N <= 512
-  // always one CTA of 8 points per thread, N = 1024 beyond that (2 rows per SM
-  // in 3.4 us either way, one in 2.0 against 3.4).
+  // First-order rows on the kernels of 8 points per thread where spread_choice
+  // takes the bucket's rows: N >= 8192 whatever the others occupy (a row's SM time
+  // on 16 SMs is about that on the split bands: 8192 24 against 22 SM us per
+  // step at full load, 16384 71 against 78, and its latency half), N = 1024 to
+  // 4096 while the whole active set fits the GPU that way (16 SMs counted for a
+  // row of 2048 or 4096, 8 for one of 1024); N <= 512 on one CTA each, N = 1024
+  // beyond that too (2 rows per SM in 3.4 us either way, one in 2.0 against 3.4).
   int spread = 0;
   if (fp32 && !forced_16() && (logn <= 10 || logn >= kSplitLogN ||
                                                    spread_demand(s) <= s.sm_count)) {
@@ -447,12 +448,17 @@ int launch_batch(Server& s, Bucket& b) {
     if (spread && logn == 10 && spread_demand(s) > s.sm_count)
       spread = rows <= spread_capacity(10, kOneCta, BPM_SPLIT_FIRST_ORDER) ? kOneCta : 0;
   }
-  size_t limit = b.members.size();
+  // the batch's requests: within what its form keeps resident, and of those on
+  // the spread kernels within theirs (the other splittings' groups march apart)
+  size_t limit = b.members.size(), spread_left = limit;
   if (fp32) {
     const bool cluster = layout < 0 && 2 * int(b.members.size()) <= s.sm_count;
-    limit = size_t(std::max(1, spread ? spread_capacity(logn, spread, BPM_SPLIT_FIRST_ORDER)
-                               : layout == kLayoutSplit4 ? fused_split4_capacity()
-                                                         : fused_launch_capacity(logn, cluster)));
+    limit = size_t(std::max(1, layout == kLayoutSplit4 ? fused_split4_capacity()
+                                                       : fused_launch_capacity(logn, cluster)));
+    if (spread) {
+      spread_left = size_t(std::max(1, spread_capacity(logn, spread, BPM_SPLIT_FIRST_ORDER)));
+      limit = std::max(limit, spread_left);
+    }
     // rows of the splitting forms march on their own kernels (N <= 4096: one
     // CTA per row, on the half-step or the fourth-order form; N = 8192,
     // 16384: the split-band cluster forms); a batch holding any stays
@@ -471,10 +477,18 @@ int launch_batch(Server& s, Bucket& b) {
   std::vector<RowDescF32> rows;
   cudaMemsetAsync(bt.d_status, 0, sizeof(int), b.st);
   const size_t nm = b.members.size();
+  size_t held = nm;   // the first request left out for the spread kernels' sake
   for (size_t k = 0; k < nm && bt.items.size() < limit; ++k) {
     ReqPtr r = b.members[(b.rr + k) % nm];
     bpm_plan_s* p = r->plan;
     if (r->failed != BPM_OK || r->n_sched >= p->nz) continue;
+    if (spread && p->split == BPM_SPLIT_FIRST_ORDER) {
+      if (spread_left == 0) {
+        if (held == nm) held = (b.rr + k) % nm;
+        continue;
+      }
+      --spread_left;
+    }
     if (r->ready) {   // first batch of this request: wait for its staging
       cudaStreamWaitEvent(b.st, r->ready, 0);
       cudaEventDestroy(r->ready);
@@ -495,7 +509,7 @@ int launch_batch(Server& s, Bucket& b) {
     auto& g = groups[3 * steps + p->split];
     g.insert(g.end(), rows.begin(), rows.end());
   }
-  b.rr = nm ? (b.rr + bt.items.size()) % nm : 0;
+  b.rr = held < nm ? held : nm ? (b.rr + bt.items.size()) % nm : 0;
   if (bt.err == BPM_OK && !groups.empty()) {
     size_t total = 0;
     for (auto& kv : groups) total += kv.second.size();
@@ -739,7 +753,8 @@ int bpm_submit(bpm_plan_t plan, const double* psi_in, double* psi_out, void* rec
     return fail(BPM_ERR_INVALID, "plan, psi_in, psi_out and out must be non-NULL");
   *out = 0;
   if (plan->ny > 1) return fail(BPM_ERR_INVALID, "the server takes 2D plans only");
-  // (Forest-Ruth at nx = 16384 marches stage by stage: not in a shared launch)
+  // (Forest-Ruth at nx = 16384 has no shared launch: stage by stage beyond the
+  // spread kernels' rows, and splitting groups march on the kernels before those)
   if (plan->precision == BPM_FP32_FUSED && plan->split == BPM_SPLIT_FOREST_RUTH &&
       plan->logn > kSplitLogN)
     return fail(BPM_ERR_INVALID, "the server marches FP32 Forest-Ruth plans up to nx = 8192");

@@ -49,3 +49,28 @@ def test_final_powers_of_a_request_and_a_device_march(bpm_lib, nx, rows, nz):
             assert np.array_equal(pw.cpu().numpy(), dev_alone)
             assert np.array_equal(y.cpu().numpy(), field_alone)
             assert np.array_equal(p, srv_alone) and np.array_equal(out, out_alone)
+
+
+def test_spread_rows_beside_another_splitting(bpm_lib, monkeypatch):
+    """More first-order requests of 8192 than the spread kernel keeps resident (14)
+    share their bucket with Forest-Ruth ones, which march apart and are not counted
+    against that: every request equals its march alone, whatever kernels the two
+    took: 20 steps of Forest-Ruth's three propagations on either side, one rounding
+    each (2 * 60 * 2^-24 = 7.2e-6)."""
+    monkeypatch.delenv("BPM_FUSED_LAYOUT", raising=False)
+    binding.bpm_server_configure(0.6, 64, 8, 1000)
+    rng = np.random.default_rng(8)
+    items = []
+    for i in range(22):
+        wl = inputs.serving_request(rng, 8192, 20)
+        split = binding.BPM_SPLIT_FOREST_RUTH if i % 4 == 3 else binding.BPM_SPLIT_FIRST_ORDER
+        plan = binding.Plan(wl, binding.BPM_FP32_FUSED, splitting=split)
+        items.append((plan, wl, np.empty_like(wl.psi0)))
+    tickets = [binding.bpm_submit(plan.handle, wl.psi0, out) for plan, wl, out in items]
+    for t in tickets:
+        assert binding.bpm_poll(t, -1) == binding.BPM_OK
+    binding.bpm_server_configure(0.6, 64, 256, 1000)
+    for plan, wl, out in items:
+        alone = plan.propagate(records=False, powers=False).psi
+        assert np.linalg.norm(out - alone) <= 7.2e-6 * np.linalg.norm(alone)
+        plan.close()
