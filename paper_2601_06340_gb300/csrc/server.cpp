@@ -73,7 +73,7 @@ struct Request {
   void* d_state = nullptr;     // c64 (FP32); FP64 requests march in their plan's state
   void* d_rec = nullptr;
   double* d_pow = nullptr;
-  double2* d_g = nullptr;
+  double2* d_g = nullptr;      // phase factors; behind them
   void* d_fin = nullptr;       // launch_finish scratch (the plan's may be in use by a march
                                // of the plan on a caller's stream)
   double2* d_out = nullptr;    // c128 staging
@@ -198,7 +198,7 @@ void release(Server& s, Request& r) {
     cudaEventDestroy(r.ready);
     r.ready = nullptr;
   }
-  void* ptrs[] = {r.d_state, r.d_rec, r.d_pow, r.d_g, r.d_fin, r.d_out};
+  void* ptrs[] = {r.d_state, r.d_rec, r.d_pow, r.d_g, r.d_out};
   for (void* p : ptrs)
     if (p) cudaFreeAsync(p, s.io_stream);
   r.d_state = r.d_rec = nullptr;
@@ -233,9 +233,9 @@ int admit_device(Server& s, Request& r) {
   if (p->precision == BPM_FP32_FUSED) A(&r.d_state, nb * 2 * n * cs);
   if (r.records && p->n_rec > 0) A(&r.d_rec, nb * size_t(p->n_rec) * 2 * n * cs);
   A(reinterpret_cast<void**>(&r.d_pow), nb * size_t(p->n_rec + 1) * 2 * 8);
-  A(reinterpret_cast<void**>(&r.d_g), nb * 16);
   const size_t fin_bytes = finish_scratch_bytes(p->nb, p->nx);
-  A(&r.d_fin, fin_bytes);
+  A(reinterpret_cast<void**>(&r.d_g), nb * 16 + fin_bytes);
+  r.d_fin = r.d_g + nb;
   A(reinterpret_cast<void**>(&r.d_out), nb * 2 * n * 16);
   if (e == cudaSuccess) e = cudaMemsetAsync(r.d_fin, 0, fin_bytes, st);
   if (e != cudaSuccess) {
