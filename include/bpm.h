@@ -216,15 +216,16 @@ int bpm_propagate(bpm_plan_t plan, const double* psi_in, double* psi_out,
  * [B][n_rec+1][2] or NULL.  The call returns after enqueueing; the caller
  * synchronises the stream before reading outputs or freeing inputs.
  * Marches of one plan share its device scratch (row descriptors, phase
- * factors, the FP64 state): enqueue them on one stream, or order the
- * streams.  An expired bounded wait inside a march is reported by
+ * factors, the final powers' partial sums, the FP64 state): enqueue them on one
+ * stream, or order the streams.  (A request of an FP32 plan that bpm_submit takes
+ * meanwhile has scratch of its own.)  An expired bounded wait inside a march is reported by
  * bpm_device_status (or by the plan's next bpm_propagate).  Graph capture:
  * FP32 plans (2D and 3D) may be captured into a CUDA graph once they have
  * marched outside a capture (strain slices prepared, schedule buffers
  * sized); the march's per-call uploads then travel as kernel parameters,
  * so a replay repeats the captured march (same buffers, steps and launch
  * shape -- the fixed rule's).  While `stream` is capturing, FP64 plans,
- * Forest-Ruth plans that march stage by stage (nx = 16384, or 8192 with
+ * Forest-Ruth plans of nx = 16384 (or 8192 with
  * BPM_FUSED_LAYOUT=staged) and plans not yet marched return BPM_ERR_INVALID
  * and enqueue nothing. */
 int bpm_propagate_device(bpm_plan_t plan, const void* d_psi_in,

@@ -1353,11 +1353,12 @@ int bpm_propagate_device(bpm_plan_t plan, const void* d_psi_in, void* d_psi_out,
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // Under graph capture the march's per-call uploads go through kernel
   // parameters (see upload); what cannot be captured is refused before
-  // anything is enqueued: FP64 plans (their march uploads per-record phase
-  // factors and swaps buffers on the host), Forest-Ruth plans that march
-  // stage by stage (their schedule is uploaded in chunks from the host) and
-  // plans whose strain slices still have to be prepared (allocation and a
-  // host wait).
+  // anything is enqueued: FP64 plans (the march of nx < 64 uploads per-record
+  // phase factors and swaps buffers on the host; the one launch of larger nx
+  // could be captured, but the entry point refuses the precision as a whole),
+  // Forest-Ruth plans of nx = 16384 and staged ones (where they march stage by
+  // stage their schedule is uploaded in chunks from the host) and plans whose
+  // strain slices still have to be prepared (allocation and a host wait).
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaError_t ce = cudaStreamIsCapturing(st, &cs);
   if (ce != cudaSuccess) return cuda_fail(ce, "stream capture status");

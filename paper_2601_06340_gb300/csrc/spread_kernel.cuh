@@ -12,9 +12,9 @@
 // bands run on C SMs.  Per first-order step, single rows, against those forms:
 // N = 1024 1.82 -> 1.20 us, 4096 2.62 -> 1.40, 8192 4.97 -> 1.76, 16384 7.1 ->
 // 3.04 (all sizes and row counts: spread_choice in spread.cu).  At N = 4096,
-// C = 16 a warp issues about 980 instructions a step on 34 % of the cycles;
-// the rest waits on the exchanges (0.64 of 2.9 cycles per instruction) and on
-// its own previous results (0.67).
+// C = 16 a warp issues 929 instructions a step on 32 % of the cycles; the rest
+// waits on the exchanges and the slice (0.71 of 3.1 cycles per instruction), on
+// its own previous results (0.71) and in the poll loops (0.23).
 //
 // Layout.  N = N1 N2, x index n = n1 N2 + n2, frequency k = k1 + N1 k2:
 //   X[k1 + N1 k2] = sum_n2 W_N^(n2 k1) W_N2^(n2 k2) sum_n1 W_N1^(n1 k1) x[n].
