@@ -430,13 +430,14 @@ void twiddle_table_f32(int n, std::vector<float4>* out) {
   for (int m = 0; m <= n / 8; ++m) {
     double c, s;
     unit_root(m, n, &c, &s);
-    // of the floats next to (c, s), the pair whose error is smallest, the phase's
-    // weighted with 0.03: a forward and an inverse pass multiply by W and its
-    // conjugate, so the modulus error is the one that repeats every step at the
-    // same modes, while a single step sees both.  Relative error of the spread
-    // kernels, geometric means over nx = 256 .. 16384, against the modulus alone:
-    // one far-field step 1.07 -> 1.05 times the two-pass kernels', marches of 40 to
-    // 2000 steps 1.020 -> 1.016; nearest floats 1.08, 1.034
+    // of the floats next to (c, s), the pair whose modulus is nearest to one:
+    // a forward and an inverse pass multiply by W and its conjugate, so the
+    // modulus error is the one that repeats every step at the same modes
+    // (marches of 2000-6000 steps with the spread kernels' three twiddle
+    // passes: relative error 4.7e-6 -> 4.3e-6 at N = 8192, 3.6e-6 -> 3.1e-6 at
+    // 2048).  Weighing the phase error with 0.03 made single steps 2 % better and
+    // marches of 4000 to 6000 steps 4 to 5 % worse; launches of few steps apply
+    // the low part too (kFewSteps)
     float ch = float(c), sh = float(s);
     if (m != 0 && m != n / 8) {
       const float c0 = ch, s0 = sh;
@@ -445,9 +446,7 @@ void twiddle_table_f32(int n, std::vector<float4>* out) {
         for (int j = -1; j <= 1; ++j) {
           const float ci = i == 0 ? c0 : std::nextafterf(c0, i * 2.f);
           const float sj = j == 0 ? s0 : std::nextafterf(s0, j * 2.f);
-          const double dm = 0.5 * (double(ci) * ci + double(sj) * sj - 1.0);
-          const double dp = double(sj) * c - double(ci) * s;
-          const double err = dm * dm + 0.03 * dp * dp;
+          const double err = std::fabs(double(ci) * ci + double(sj) * sj - 1.0);
           if (err < best) {
             best = err;
             ch = ci;
