@@ -26,7 +26,11 @@
 // many fit an SM; nothing but the spectra is left to read after a barrier
 // (slice, field and propagator are in flight before it).  Per step 512 x 256
 // 9.6 -> 7.2 us (of 7500 clocks a phase 3000 are the barrier, 950 the first
-// reads), 256 x 256 8.6 -> 5.8, 1024 x 512 22.3 -> 19.0, 4096 x 256 unchanged.
+// reads), 256 x 256 8.6 -> 5.8, 1024 x 512 22.3 -> 19.0.  Lines of 4096 points take
+// CTAs of 1024 threads, whose 64 registers do not hold what is in flight over a
+// barrier: read where it is used it left 70 to 130 bytes of spills instead of 600
+// to 680, and 4096 x 256 takes 48.2 (two launches) -> 36.8 us (51.2 with the spills),
+// 4096 x 1024 195 -> 154, Verlet 61.2 -> 38.8 and 269 -> 165.
 #pragma once
 
 #include "fused4s_kernel.cuh"
@@ -69,6 +73,7 @@ struct VolCfg {
   static constexpr int TX = NX / 8, TY = NY / 8, COLS = 4;
   static constexpr int THREADS = 2 * TX > COLS * TY ? 2 * TX : COLS * TY;
   static constexpr int MINCTAS = THREADS < 512 ? 512 / THREADS : 1;   // 16 warps per SM
+  static constexpr bool HOLD = THREADS <= 512;
   static constexpr int ROWS = THREADS / (2 * TX), TILES = THREADS / (COLS * TY);
   // column stride 4 mod 16: the tile copies (4 rows x 4 columns per
   // half-warp) touch 16 bank pairs
@@ -203,38 +208,50 @@ __global__ void __launch_bounds__((VolCfg<LX, LY>::THREADS), (VolCfg<LX, LY>::MI
   const int first = blockIdx.x;
 
   float2 v[8];
+  // what a phase reads besides the spectra, in flight over the barrier before it
+  // (with the 64 registers of a 1024-thread CTA, Nx = 4096, read where it is used)
+  constexpr bool HOLD = C::HOLD;
   float2 org[8], e0[8], e1[8];      // row phase: field and slices of the first item
   float2 pr[8];                     // column phase: propagator of the first item
   auto line_off = [&](int item) {   // offset of this thread's line and band
     const int line = item * C::ROWS + rslot;
     return (size_t(line / NY) * 2 + rband) * PLANE + size_t(line % NY) * NX + rt;
   };
-  auto slice = [&](int item, int n, float2* e) {
+  auto slice_at = [&](int item, int n) {
     const int y = (item * C::ROWS + rslot) % NY;
-    const float2* ph = p.phasor + size_t(n) * PLANE + size_t(y) * NX + rt;
+    return p.phasor + size_t(n) * PLANE + size_t(y) * NX + rt;
+  };
+  auto slice = [&](int item, int n, float2* e) {
+    const float2* ph = slice_at(item, n);
 #pragma unroll
     for (int j = 0; j < 8; ++j) e[j] = __ldg(&ph[j * TX]);
   };
   auto row_fetch = [&](int item, int n, bool next) {
+    if constexpr (!HOLD) return;
     const float2* o = p.org + line_off(item);
 #pragma unroll
     for (int j = 0; j < 8; ++j) org[j] = __ldcg(&o[j * TX]);
     slice(item, n, e0);
     if (half && next) slice(item, n + 1, e1);
   };
+  auto prop_at = [&](int item) {
+    return p.prop + size_t(item * C::TILES + cslot) * (COLS * NY) + cin;
+  };
   auto col_fetch = [&](int item) {
-    const float2* t = p.prop + size_t(item * C::TILES + cslot) * (COLS * NY) + cin;
+    if constexpr (!HOLD) return;
+    const float2* t = prop_at(item);
 #pragma unroll
     for (int j = 0; j < 8; ++j) pr[j] = __ldg(&t[j * COLS * TY]);
   };
-  auto couple = [&](int item, const float2* e, const float2* coup) {
+  auto couple = [&](int item, int n, const float2* e, const float2* coup) {   // e: slice n
     const int r = (item * C::ROWS + rslot) / NY;
+    const float2* ph = slice_at(item, n);
     const float2 am1 = __ldg(&coup[2 * r]), bb = __ldg(&coup[2 * r + 1]);
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const float2 q = make_float2(__shfl_xor_sync(0xffffffffu, v[j].x, 16),
                                    __shfl_xor_sync(0xffffffffu, v[j].y, 16));
-      v[j] = couple_cell(v[j], q, e[j], rband, am1, bb);
+      v[j] = couple_cell(v[j], q, HOLD ? e[j] : __ldg(&ph[j * TX]), rband, am1, bb);
     }
   };
   auto put_line = [&](float2* to, int item) {
@@ -246,10 +263,11 @@ __global__ void __launch_bounds__((VolCfg<LX, LY>::THREADS), (VolCfg<LX, LY>::MI
   __syncthreads();      // (tables)
   for (int item = first; item < row_items; item += gridDim.x) {
     row_fetch(item, p.n_begin, false);
+    const float2* o = p.org + line_off(item);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = org[j];
+    for (int j = 0; j < 8; ++j) v[j] = HOLD ? org[j] : __ldcg(&o[j * TX]);
     if (half) {         // the launch's first half-step, on the slice of its first step
-      couple(item, e0, p.coup_half);
+      couple(item, p.n_begin, e0, p.coup_half);
       put_line(p.org, item);
     }
     if (item != first) __syncthreads();   // (the previous item's reads of the lines)
@@ -283,8 +301,12 @@ __global__ void __launch_bounds__((VolCfg<LX, LY>::THREADS), (VolCfg<LX, LY>::MI
       __syncthreads();
       vol_get<LY, 0>(cbuf, v, ct);
       vol_fwd<LY>(v, cbuf, twy, ct);
+      const float2* t = prop_at(item);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = cmul_f(v[j], pr[j].x, pr[j].y);
+      for (int j = 0; j < 8; ++j) {
+        const float2 d = HOLD ? pr[j] : __ldg(&t[j * COLS * TY]);
+        v[j] = cmul_f(v[j], d.x, d.y);
+      }
       vol_inv<LY>(v, cbuf, twy, ct);
       vol_put<LY, 0>(cbuf, v, ct);
       __syncthreads();
@@ -310,9 +332,10 @@ __global__ void __launch_bounds__((VolCfg<LX, LY>::THREADS), (VolCfg<LX, LY>::MI
       }
       vol_inv<LX>(v, rbuf, twx, rt);
       // psi_p = psi + increment, then the coupling with the other band (lane ^ 16)
+      const float2* o = p.org + line_off(item);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = cadd(org[j], v[j]);
-      couple(item, e0, half ? p.coup_half : p.coup);
+      for (int j = 0; j < 8; ++j) v[j] = cadd(HOLD ? org[j] : __ldcg(&o[j * TX]), v[j]);
+      couple(item, n, e0, half ? p.coup_half : p.coup);
       if (rec) {
         const int line = item * C::ROWS + rslot, r = line / NY, y = line % NY;
         const int slot = (n + 1) / p.record_every - 1;
@@ -342,7 +365,7 @@ __global__ void __launch_bounds__((VolCfg<LX, LY>::THREADS), (VolCfg<LX, LY>::MI
           __syncthreads();
         }
       }
-      if (half && !last) couple(item, e1, p.coup_half);   // the next step's first half
+      if (half && !last) couple(item, n + 1, e1, p.coup_half);   // the next step's first half
       put_line(p.org, item);
       if (!last) {
         vol_fwd<LX>(v, rbuf, twx, rt);
