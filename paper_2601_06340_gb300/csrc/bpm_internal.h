@@ -332,7 +332,8 @@ int launch_stage(const MarchInput& in, void* dst, void* d_a, const void* a, size
                  void* d_b, const void* b, size_t bytes_b, cudaStream_t st);
 bool stage_fits(size_t bytes_a, size_t bytes_b);
 // out = state * g per row and, if final_powers, the lines' powers; scratch of
-// finish_scratch_bytes, zero at its first use.
+// finish_scratch_bytes (16-byte aligned or behind 16 bytes a row), whose first
+// finish_count_bytes, the lines' counters, are zero at its first use.
 int launch_finish_f32(const float2* state, double2* out_c128, float2* out_c64,
                       const double* gphase, int n_rows, int nx, double dx, double* final_powers,
                       int power_stride, void* scratch, cudaStream_t st);
@@ -340,6 +341,7 @@ int launch_finish_f64(const double2* state, double2* out, const double* gphase, 
                       int nx, double dx, double* final_powers, int power_stride, void* scratch,
                       cudaStream_t st);
 size_t finish_scratch_bytes(int n_rows, int nx);
+size_t finish_count_bytes(int n_rows);
 int launch_omega_to_t(const void* d_in, void* d_out, int nb, int nx,
                       int precision, cudaStream_t st);
 int fused_smem_bytes(int logn);

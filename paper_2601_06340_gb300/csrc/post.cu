@@ -98,8 +98,8 @@ template <typename TIn>
 int launch_finish(const TIn* state, double2* out128, float2* out64, const double* g, int n_rows,
                   int nx, double dx, double* pw, int pw_stride, void* scratch, cudaStream_t st) {
   const int blocks = finish_blocks(n_rows, nx), lines = 2 * n_rows;
-  double* part = static_cast<double*>(scratch);
-  unsigned* count = reinterpret_cast<unsigned*>(part + size_t(lines) * blocks);
+  unsigned* count = static_cast<unsigned*>(scratch);
+  double* part = reinterpret_cast<double*>(count + lines);   // (an even number of lines)
   const double2* g2 = reinterpret_cast<const double2*>(g);
   const unsigned grid = unsigned(lines) * unsigned(blocks);
   if (finish_per(n_rows, nx) == 1)
@@ -186,8 +186,10 @@ int launch_convert_in(const double2* src, float2* dst, size_t n, cudaStream_t st
   return e == cudaSuccess ? BPM_OK : cuda_fail(e, "convert input");
 }
 
+size_t finish_count_bytes(int n_rows) { return size_t(2 * n_rows) * sizeof(unsigned); }
+
 size_t finish_scratch_bytes(int n_rows, int nx) {
-  return size_t(2 * n_rows) * (size_t(finish_blocks(n_rows, nx)) * sizeof(double) + sizeof(unsigned));
+  return finish_count_bytes(n_rows) + size_t(2 * n_rows) * finish_blocks(n_rows, nx) * sizeof(double);
 }
 
 int launch_finish_f32(const float2* state, double2* out_c128, float2* out_c64,

@@ -180,11 +180,14 @@ void pinned_put(Server& s, void* p, size_t bytes) {
   if (p) s.pinned_pool[bytes].push_back(p);
 }
 
-// Pinned staging of a request: [psi c128][records][powers].
-size_t stage_bytes(const bpm_plan_s* p, bool rec) {
+// Pinned staging of a request: [psi c128][records][powers], and room behind that
+// for the phase factors with the finish counters to start at the powers.
+size_t powers_at(const bpm_plan_s* p, bool rec) {
   const size_t n = p->nx, nb = p->nb, cs = csize_of(p);
-  return nb * 2 * n * 16 + (rec ? nb * size_t(p->n_rec) * 2 * n * cs : 0) +
-         nb * size_t(p->n_rec + 1) * 2 * 8;
+  return nb * 2 * n * 16 + (rec ? nb * size_t(p->n_rec) * 2 * n * cs : 0);
+}
+size_t stage_bytes(const bpm_plan_s* p, bool rec) {
+  return powers_at(p, rec) + p->nb * size_t(p->n_rec + 1) * 2 * 8 + finish_count_bytes(p->nb);
 }
 
 void release(Server& s, Request& r) {
@@ -233,11 +236,9 @@ int admit_device(Server& s, Request& r) {
   if (p->precision == BPM_FP32_FUSED) A(&r.d_state, nb * 2 * n * cs);
   if (r.records && p->n_rec > 0) A(&r.d_rec, nb * size_t(p->n_rec) * 2 * n * cs);
   A(reinterpret_cast<void**>(&r.d_pow), nb * size_t(p->n_rec + 1) * 2 * 8);
-  const size_t fin_bytes = finish_scratch_bytes(p->nb, p->nx);
-  A(reinterpret_cast<void**>(&r.d_g), nb * 16 + fin_bytes);
+  A(reinterpret_cast<void**>(&r.d_g), nb * 16 + finish_scratch_bytes(p->nb, p->nx));
   r.d_fin = r.d_g + nb;
   A(reinterpret_cast<void**>(&r.d_out), nb * 2 * n * 16);
-  if (e == cudaSuccess) e = cudaMemsetAsync(r.d_fin, 0, fin_bytes, st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return e == cudaErrorMemoryAllocation ? BPM_ERR_OOM : BPM_ERR_CUDA;
@@ -270,11 +271,13 @@ int retire_enqueue(Server& s, Request& r) {
   std::vector<double2> g;
   phase_factors(p, p->nz, &g);
   cudaStream_t st = s.out_stream;
-  double2* hg = reinterpret_cast<double2*>(
-      static_cast<char*>(r.h_stage) + r.h_stage_bytes - nb * size_t(p->n_rec + 1) * 2 * 8);
-  // phase factors go through the (not yet used) powers area of the staging
+  char* hg = static_cast<char*>(r.h_stage) + powers_at(p, r.d_rec != nullptr);
+  // phase factors and the finish's zeroed counters go through the (not yet used)
+  // powers area of the staging
+  const size_t zero = finish_count_bytes(p->nb);
   std::memcpy(hg, g.data(), nb * 16);
-  cudaError_t e = cudaMemcpyAsync(r.d_g, hg, nb * 16, cudaMemcpyHostToDevice, st);
+  std::memset(hg + nb * 16, 0, zero);
+  cudaError_t e = cudaMemcpyAsync(r.d_g, hg, nb * 16 + zero, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return BPM_ERR_CUDA;
   const int pw_stride = 2 * (p->n_rec + 1);
   int rc;
